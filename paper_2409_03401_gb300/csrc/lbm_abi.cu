@@ -273,9 +273,17 @@ int read_mode(const lbm_ctx* c) {
     if (c->L.two) return lbm::kModePull;
     return (c->t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven;
 }
-// z planes one block of the fused flow kernel marches through (measured best of 16..128 at 512^3)
-constexpr int kZChunk = 32;
-int zchunk_of(const lbm_params* p) { return p->nz < kZChunk ? p->nz : kZChunk; }
+// Whether a flow step of the two-buffer layout runs as the fused kernel: FP32 storage from
+// 600,000 nodes on, and slabs (whose ghost phi it reads in place). The others take a phi pass and
+// the per-node pull step, the same fields bit for bit. The fused kernel computes phi of its halo
+// again (a third more): that saves HBM traffic, but 16-bit and FP64 storage pay for it in issue
+// slots and on the FP64 pipe (512^3 FP16 8.01 ms against 7.29 for the two passes, 64^3 27 against
+// 21 us; FP64 128^3 2.45 against 2.16 ms), and in lattices that stay in L2 its planes, one after
+// another, take longer than two launches (FP32 64^3 24 against 18 us, 80^3 44 against 43 us,
+// 96^3 61 against 68 us).
+bool one_pass(const lbm_ctx* c) {
+    return c->L.two && fused_flow(&c->p) && (c->slab || (c->p.storage == LBM_F32 && c->L.n >= 600000));
+}
 
 }  // namespace
 
@@ -342,14 +350,14 @@ void launch_one(lbm_ctx* c, int64_t t, cudaEvent_t* e) {
     // src holds time level t; dst receives t + 1 (the same buffer in the in-place layout)
     const StateView& src = (c->L.two && (t & 1)) ? c->st1 : c->st;
     const StateView& dst = c->L.two ? ((t & 1) ? c->st : c->st1) : c->st;
-    const bool fused = c->L.two && fused_flow(&c->p);
+    const bool fused = one_pass(c);
     if (c->p.flow && !fused) {
         LBM_DISPATCH(c->p.storage, launch_phi, c->dp, src, c->p.lattice, mode, c->work + c->L.off_phi, c->stream);
         if (c->slab) ghost_phi_to_field(c);
     }
     if (e) cudaEventRecord(e[1], c->stream);
     if (fused) {
-        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, zchunk_of(&c->p), c->stream);
+        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, c->stream);
     } else {
         LBM_DISPATCH(c->p.storage, launch_step, c->dp, src, dst, c->p.lattice, c->p.flow != 0, mode,
                      c->work + c->L.off_phi, c->stream);
@@ -449,7 +457,7 @@ lbm_status lbm_profile_end(lbm_ctx* c, double* out) {
 }
 
 int lbm_kernels_per_step(const lbm_ctx* c) {
-    return c ? ((c->p.flow && !(c->L.two && fused_flow(&c->p))) ? 2 : 1) : 0;
+    return c ? ((c->p.flow && !one_pass(c)) ? 2 : 1) : 0;
 }
 
 int64_t lbm_time(const lbm_ctx* c) { return c ? c->t : -1; }
@@ -506,7 +514,7 @@ lbm_status lbm_step_buffers(const lbm_params* p, const void* d_src, void* d_dst,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaGetLastError();
     if (L.two && fused_flow(p)) {
-        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, zchunk_of(p), s);
+        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, s);
     } else {
         const int mode = L.two ? lbm::kModePull : ((t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven);
         char* phi = static_cast<char*>(d_work) + L.off_phi;

@@ -1236,6 +1236,20 @@ reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::t
     }
 }
 
+// Planes (rows, in 2D) a marching block goes through: the count, at most 32, for which the
+// waves of blocks over the chip's ``slots`` times the planes each block computes, ``extra`` for
+// the planes around the chunk among them, are fewest.
+inline int march_chunk(long long tiles, int n, long long slots, double extra) {
+    int best = 1;
+    double cost = 1e300;
+    for (int c = 1; c <= n && c <= 32; ++c) {
+        const long long blocks = tiles * ((n + c - 1) / c);
+        const double t = double((blocks + slots - 1) / slots) * (c + extra);
+        if (t <= cost) { cost = t; best = c; }
+    }
+    return best;
+}
+
 // ------------------------------------------------------------------------------------
 // Host launchers for one storage type. ``mode`` is AA_EVEN / AA_ODD for the in-place
 // layout and PULL for the two-buffer layout (st = the current state buffer).
@@ -1290,8 +1304,10 @@ struct Launchers {
         }
         LBM_MODE_SWITCH(mode, step_kernel<T, LAT, FLOW, M, -1><<<grid, bx, 0, s>>>(P, st, out, phi));
     }
-    static void fused(const DevParams& P, const StateView& src, const StateView& dst, int zchunk, cudaStream_t s) {
+    static void fused(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
         const dim3 block(FX, FY);
+        const int zchunk = march_chunk((long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY), P.z_hi - P.z_lo,
+                                       152 * fused_min_blocks<T, 0>(), 0.7);
         const dim3 grid((P.nx + FX - 1) / FX, (P.ny + FY - 1) / FY, (P.z_hi - P.z_lo + zchunk - 1) / zchunk);
         constexpr size_t smem = fused_smem_bytes<T>();
         // instances per flow collision (see fused_flow_kernel)
@@ -1408,9 +1424,9 @@ struct Launchers {
         else if (flow) Launchers<T>::step<LAT_D3Q7, true>(P, st, out, mode, phi, s);                       \
         else Launchers<T>::step<LAT_D3Q7, false>(P, st, out, mode, phi, s);                                \
     }                                                                                                     \
-    void launch_fused_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst, int zchunk, \
+    void launch_fused_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst,            \
                                cudaStream_t s) {                                                          \
-        Launchers<T>::fused(P, src, dst, zchunk, s);                                                      \
+        Launchers<T>::fused(P, src, dst, s);                                                              \
     }                                                                                                     \
     void launch_fields_##SUFFIX(const DevParams& P, const StateView& st, int lat, bool flow, int mode,    \
                                 void* phi, FieldPtrs out, cudaStream_t s) {                               \

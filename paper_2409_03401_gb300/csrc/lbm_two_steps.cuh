@@ -1,0 +1,264 @@
+// Two steps without flow in one pass over memory (no-flow D2Q5, D2Q9 and D3Q7 lattices).
+// Reads the populations of an even time level t of the in-place layout (slot k of node x
+// holds the incoming population k) from ``src`` and writes time level t + 2, in the same
+// layout, to ``dst``: the first collision's results travel one node through registers,
+// shuffles and (3D, along y) shared memory instead of through HBM. The arithmetic of a node
+// is collide_at_rest in both steps, so the result equals two calls of step_kernel bit for bit.
+#pragma once
+
+namespace lbm {
+
+__device__ __forceinline__ float from_left(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ float from_right(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+template <class T, int LAT>
+__device__ __forceinline__ Node<T, LAT, false> load_node(const StateView& src, int node, const DevParams& P) {
+    Addr<AA_EVEN> ad;
+    ad.self = node;
+    Node<T, LAT, false> nd;
+    nd.gather_scalars(src, ad, P);
+    return nd;
+}
+
+// First collision of a node.
+template <class T, int LAT>
+__device__ __forceinline__ void collide_first(Node<T, LAT, false> nd, const DevParams& P,
+                                              typename RealOf<T>::type (&out)[3][Scalar<LAT>::Q]) {
+    using R = typename RealOf<T>::type;
+    nd.moments(P);
+    collide_at_rest<T, LAT>(nd, P, [&](int set, int k, R r) {
+        out[set - SET_G][k] = r;
+        return r;
+    });
+}
+
+// Second collision of every lane's node, incoming populations in[set][k], and the store of
+// what comes in at each inner lane's node next: populations moving along x come from the lane
+// beside, or, behind a wall (lo: x = -1, hi: x = nx), from the node itself (bounce-back), so that
+// a warp stores whole rows at its own x. ``to(k)`` is the slot for population k of this x.
+template <class T, int LAT, class To>
+__device__ __forceinline__ void collide_second(const typename RealOf<T>::type (&in)[3][Scalar<LAT>::Q],
+                                               const StateView& dst, int self, bool inner, bool lo, bool hi,
+                                               const DevParams& P, To to) {
+    using R = typename RealOf<T>::type;
+    using L = Scalar<LAT>;
+    Node<T, LAT, false> nd;
+#pragma unroll
+    for (int k = 0; k < L::Q; ++k) {
+        nd.g[k] = in[0][k];
+        nd.hA[k] = in[1][k];
+        nd.hB[k] = in[2][k];
+    }
+    nd.moments(P);
+    T held[3];
+    collide_at_rest<T, LAT>(nd, P, [&](int set, int k, R r) {
+        if (k == 0) {
+            if (inner) store_rest_at<T, LAT>(dst, set, self, r, P);
+            return r;
+        }
+        if (k & 1) {
+            held[set - SET_G] = r;                                     // stored with its opposite
+        } else {
+            T a = held[set - SET_G], b = r;                            // moving along e_{k-1} and back
+            if (L::ex(k - 1) != 0) {
+                const bool fwd = L::ex(k - 1) > 0;
+                const T ma = fwd ? from_left(a) : from_right(a), mb = fwd ? from_right(b) : from_left(b);
+                const T oa = a;
+                a = (fwd ? lo : hi) ? b : ma;
+                b = (fwd ? hi : lo) ? oa : mb;
+            }
+            if (inner) {
+                store_at<T, LAT>(dst, set, k - 1, to(k - 1), a);
+                store_at<T, LAT>(dst, set, k, to(k), b);
+            }
+        }
+        return r;
+    });
+}
+
+__device__ __forceinline__ int wrapped(int q, int n) { return ((q % n) + n) % n; }
+
+// 3D: a block of 32 x 16 threads marches along z; its 28 x 14 inner threads own nodes, the
+// outer ring computes the first collision of the tile's neighbours again.
+constexpr int T2X = 32, T2Y = 16, T2IX = T2X - 4, T2IY = T2Y - 2;
+constexpr int kTwoStepsBlocks = 2;
+
+template <class T>
+__global__ void __launch_bounds__(T2X * T2Y, kTwoStepsBlocks)
+two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst, int zchunk) {
+    begin_after_previous();
+    using R = typename RealOf<T>::type;
+    constexpr int Q = 7;
+    // populations moving along y, of three planes: the plane being assembled, the next one,
+    // and the one that threads ahead of the slowest (by one barrier) already write
+    __shared__ R ys[3][6][T2Y][T2X];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int x = int(blockIdx.x) * T2IX + tx - 2, y = int(blockIdx.y) * T2IY + ty - 1;
+    const int zs = blockIdx.z * zchunk, ze = min(zs + zchunk, P.nz);
+    // this thread's column, wrapped: lanes past the row's end read nodes whose values nobody takes
+    const int gx = wrapped(x, P.nx), gy = wrapped(y, P.ny);
+    const int nxy = P.nx * P.ny;
+    const int col = gy * P.nx + gx;
+    const bool row_in = ty >= 1 && ty <= T2IY && y < P.ny;             // whole warps
+    const bool inner = tx >= 2 && tx < T2IX + 2 && x < P.nx;
+    const bool wall_lo = P.wall_x && x == 0, wall_hi = P.wall_x && x == P.nx - 1;
+    // columns of the neighbours along y
+    const int cyp = (gy + 1 == P.ny ? 0 : gy + 1) * P.nx + gx, cym = (gy == 0 ? P.ny - 1 : gy - 1) * P.nx + gx;
+
+    R in[3][Q];      // incoming populations of plane z (second step); +z from z - 1 in slot 5
+    R up[3];         // moving +z out of plane z
+    R o[3][Q];
+    // first collision of plane zz; leaves what comes in along x in o[.][1], o[.][2] and its -z
+    // movers in o[.][6]
+    auto first = [&](int zz, int slot) {
+        const int zr = zz < 0 ? zz + P.nz : (zz >= P.nz ? zz - P.nz : zz);
+        collide_first<T, LAT_D3Q7>(load_node<T, LAT_D3Q7>(src, zr * nxy + col, P), P, o);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            ys[slot][2 * s][ty][tx] = o[s][3];
+            ys[slot][2 * s + 1][ty][tx] = o[s][4];
+            const R a = from_left(o[s][1]), b = from_right(o[s][2]), own = o[s][1];
+            o[s][1] = wall_lo ? o[s][2] : a;
+            o[s][2] = wall_hi ? own : b;
+        }
+    };
+    int slot = 0;
+    if (zs > 0 || !P.wall_z) {
+        first(zs - 1, 2);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) in[s][5] = o[s][5];
+        first(zs, slot);
+    } else {
+        first(zs, slot);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) in[s][5] = o[s][6];                // bounced at the wall
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        in[s][0] = o[s][0]; in[s][1] = o[s][1]; in[s][2] = o[s][2];
+        up[s] = o[s][5];
+    }
+    for (int z = zs; z < ze; ++z) {
+        const int next = slot == 2 ? 0 : slot + 1;
+        const bool top = P.wall_z && z == P.nz - 1, low = P.wall_z && z == 0;
+        if (!top) first(z + 1, next);
+        __syncthreads();
+        if (row_in) {
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                in[s][3] = ys[slot][2 * s][ty - 1][tx];
+                in[s][4] = ys[slot][2 * s + 1][ty + 1][tx];
+                in[s][6] = top ? up[s] : o[s][6];
+            }
+            const int zp = z + 1 == P.nz ? 0 : z + 1, zm = z == 0 ? P.nz - 1 : z - 1;
+            const int self = z * nxy + col;
+            collide_second<T, LAT_D3Q7>(in, dst, self, inner, wall_lo, wall_hi, P, [&](int k) -> Slot {
+                switch (k) {
+                    case 3: return {z * nxy + cyp, 3};
+                    case 4: return {z * nxy + cym, 4};
+                    case 5: return top ? Slot{self, 6} : Slot{zp * nxy + col, 5};
+                    case 6: return low ? Slot{self, 5} : Slot{zm * nxy + col, 6};
+                    default: return {self, k};
+                }
+            });
+        }
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            in[s][0] = o[s][0]; in[s][1] = o[s][1]; in[s][2] = o[s][2];
+            in[s][5] = up[s];
+            up[s] = o[s][5];
+        }
+        slot = next;
+    }
+}
+
+// 2D: a warp marches along y on its own; its 30 inner lanes own nodes, the outer two compute
+// the first collision of the neighbours again. No shared memory and no barrier.
+constexpr int T2Warps = 4, kTwoSteps2DBlocks = 4;
+
+template <class T, int LAT>
+__global__ void __launch_bounds__(32 * T2Warps, kTwoSteps2DBlocks)
+two_steps_2d_kernel(const DevParams P, const StateView src, const StateView dst, int ychunk) {
+    begin_after_previous();
+    using R = typename RealOf<T>::type;
+    using L = Scalar<LAT>;
+    constexpr int Q = L::Q;
+    const int lane = threadIdx.x & 31;
+    const int win = blockIdx.x * T2Warps + (threadIdx.x >> 5);
+    if (win * T2IX >= P.nx) return;                                    // whole warps
+    const int x = win * T2IX + lane - 2;
+    const int ys = blockIdx.y * ychunk, ye = min(ys + ychunk, P.ny);
+    const int gx = wrapped(x, P.nx);
+    const bool inner = lane >= 2 && lane < T2IX + 2 && x < P.nx;
+    const bool wall_lo = P.wall_x && x == 0, wall_hi = P.wall_x && x == P.nx - 1;
+
+    R in[3][Q];      // incoming populations of row y: the rows y - 1 and y filled in, y + 1 to come
+    R up[3][Q];      // of row y + 1: what row y sends up
+    R o[3][Q];
+    auto row = [&](int yy) {
+        return load_node<T, LAT>(src, (yy < 0 ? yy + P.ny : (yy >= P.ny ? yy - P.ny : yy)) * P.nx + gx, P);
+    };
+    Node<T, LAT, false> next = row(ys - 1);
+    auto first = [&](int yy) {
+        const Node<T, LAT, false> nd = next;
+        next = row(yy < ye ? yy + 1 : yy);
+        collide_first<T, LAT>(nd, P, o);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            const R p1 = o[s][1], m1 = o[s][2];                        // +x and -x, for walls
+#pragma unroll
+            for (int k = 1; k < Q; ++k) {
+                if (L::ex(k) > 0) o[s][k] = from_left(o[s][k]);
+                if (L::ex(k) < 0) o[s][k] = from_right(o[s][k]);
+            }
+            if constexpr (LAT == LAT_D2Q5) {
+                if (wall_lo) o[s][1] = m1;
+                if (wall_hi) o[s][2] = p1;
+            }
+        }
+    };
+    // hand the outputs of a row on: its own level and downward movers are consumed by now
+    auto rotate = [&]() {
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                if (L::ey(k) == 0) in[s][k] = o[s][k];
+                if (L::ey(k) > 0) { in[s][k] = up[s][k]; up[s][k] = o[s][k]; }
+            }
+    };
+    first(ys - 1);
+    rotate();
+    first(ys);
+    rotate();
+    for (int y = ys; y < ye; ++y) {
+        first(y + 1);
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+            for (int k = 0; k < Q; ++k)
+                if (L::ey(k) < 0) in[s][k] = o[s][k];
+        const int yp = y + 1 == P.ny ? 0 : y + 1, ym = y == 0 ? P.ny - 1 : y - 1;
+        collide_second<T, LAT>(in, dst, y * P.nx + gx, inner, wall_lo, wall_hi, P, [&](int k) -> Slot {
+            return {(L::ey(k) > 0 ? yp : (L::ey(k) < 0 ? ym : y)) * P.nx + gx, k};
+        });
+        rotate();
+    }
+}
+
+template <class T, int LAT>
+void launch_two_steps_at(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
+    if constexpr (LAT == LAT_D3Q7) {
+        const dim3 tiles((P.nx + T2IX - 1) / T2IX, (P.ny + T2IY - 1) / T2IY);
+        const int zc = march_chunk((long long)tiles.x * tiles.y, P.nz, 152 * kTwoStepsBlocks, 2.0);
+        launch_after_previous<float>(two_steps_3d_kernel<T>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(T2X, T2Y), 0, s, P,
+                              src, dst, zc);
+    } else {
+        const int wins = (P.nx + T2IX - 1) / T2IX, bx = (wins + T2Warps - 1) / T2Warps;
+        const int yc = march_chunk(bx, P.ny, 152 * kTwoSteps2DBlocks, 2.0);
+        launch_after_previous<float>(two_steps_2d_kernel<T, LAT>, dim3(bx, (P.ny + yc - 1) / yc), dim3(32 * T2Warps), 0, s, P, src,
+                              dst, yc);
+    }
+}
+
+}  // namespace lbm
