@@ -173,6 +173,7 @@ adjoint_step_kernel(const DevParams P, const StateView st, const typename RealOf
     using R = typename RealOf<T>::type;
     using L = Scalar<LAT>;
     constexpr int Q = L::Q;
+    begin_after_previous();
     R acc[kNAcc] = {R(0), R(0), R(0), R(0), R(0), R(0)};
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -317,12 +318,8 @@ void adjoint_step_T(const DevParams& P, const StateView& st, bool odd, const voi
     int bx;
     const dim3 grid = node_grid(P, bx);
     const double om_g_deriv = -P.om_g * P.om_g * P.inv_cs2;   // d om_g / d M_phi
-    if (odd)
-        adjoint_step_kernel<T, LAT, AA_ODD><<<grid, bx, 0, s>>>(P, st, static_cast<const R*>(lam_next),
-                                                                static_cast<R*>(lam), partials, om_g_deriv);
-    else
-        adjoint_step_kernel<T, LAT, AA_EVEN><<<grid, bx, 0, s>>>(P, st, static_cast<const R*>(lam_next),
-                                                                 static_cast<R*>(lam), partials, om_g_deriv);
+    launch_after_previous<R>(odd ? adjoint_step_kernel<T, LAT, AA_ODD> : adjoint_step_kernel<T, LAT, AA_EVEN>, grid, dim3(bx),
+                          0, s, P, st, static_cast<const R*>(lam_next), static_cast<R*>(lam), partials, om_g_deriv);
 }
 
 template <class T, int LAT>

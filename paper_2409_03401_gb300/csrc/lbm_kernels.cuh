@@ -19,6 +19,32 @@
 namespace lbm {
 
 constexpr int kBlockX = 128;
+
+// Step kernels follow one another in a stream with programmatic dependent launch: the next
+// one's blocks are set up while the last blocks of this one still run (launch_dependents, once
+// every block has started), and wait there until it has completed and its stores are visible.
+__device__ __forceinline__ void begin_after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// R: the kernel's arithmetic. FP64 kernels of more blocks than SMs are launched the plain way:
+// blocks set up early land unevenly beside those still running, and the FP64 pipe of the SMs
+// that got more decides the step (864 x 34 couple: 22.6 us a step against 12.5).
+template <class R, class... P, class... A>
+inline void launch_after_previous(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  const A&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = sizeof(R) == 4 || (long long)grid.x * grid.y * grid.z <= 152 ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
 enum { AA_EVEN = 0, AA_ODD = 1, PULL = 2 };
 
 // Wrapped neighbour coordinates of one node. c[a][1 + d] is the coordinate x_a + d along
@@ -638,6 +664,7 @@ __global__ void __launch_bounds__(kBlockX)
 step_kernel(const DevParams P, const StateView st, const StateView out,
             const typename RealOf<T>::type* __restrict__ phi_field) {
     using R = typename RealOf<T>::type;
+    begin_after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
@@ -662,6 +689,7 @@ step_kernel(const DevParams P, const StateView st, const StateView out,
 template <class T, int LAT, int MODE>
 __global__ void __launch_bounds__(kBlockX)
 phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* __restrict__ phi_out) {
+    begin_after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
@@ -739,6 +767,7 @@ constexpr int fused_min_blocks() { return sizeof(typename RealOf<T>::type) == 8 
 template <class T, int COLL, bool SLAB>
 __global__ void __launch_bounds__(FT, fused_min_blocks<T, COLL>())
 fused_flow_kernel(const DevParams P, const StateView src, const StateView dst, int zchunk) {
+    begin_after_previous();
     constexpr int kColl = (!is16<T>() && COLL != 2) ? -1 : COLL;
     using R = typename RealOf<T>::type;
     using L = Scalar<LAT_D3Q7>;
@@ -1258,6 +1287,19 @@ inline dim3 node_grid(const DevParams& P, int& bx) {
     return dim3((P.nx + bx - 1) / bx, P.ny, P.z_hi - P.z_lo);
 }
 
+// Rows of the per-node step and phi kernels: blocks of 128, 96 or 64 nodes of a row, whichever
+// leaves the fewest lanes past its end; single warps in lattices so small that each SM gets at
+// most two (512 x 8 FP64 couple: 5.2 us a step against 8.2). One row per block: with y the same for a whole block the wrap
+// tests of Nbr stay uniform (two-row blocks cost the in-place FP16 step 6 %).
+inline dim3 step_grid(const DevParams& P, int& bx) {
+    const long long n = (long long)P.nx * P.ny * (P.z_hi - P.z_lo);
+    bx = P.nx >= kBlockX ? kBlockX : (P.nx + 31) / 32 * 32;
+    for (int b : {96, 64})
+        if ((P.nx + b - 1) / b * b < (P.nx + bx - 1) / bx * bx) bx = b;
+    if (n <= 32 * 152 * 2) bx = 32;
+    return dim3((P.nx + bx - 1) / bx, P.ny, P.z_hi - P.z_lo);
+}
+
 #define LBM_MODE_SWITCH(MODE_VAR, ...)                                          \
     switch (MODE_VAR) {                                                         \
         case AA_EVEN: { constexpr int M = AA_EVEN; __VA_ARGS__; } break;        \
@@ -1276,11 +1318,18 @@ struct Launchers {
         if (pull) init_kernel<T, LAT, FLOW, PULL><<<grid, bx, 0, s>>>(P, st, phi0, cA0, cB0);
         else init_kernel<T, LAT, FLOW, AA_EVEN><<<grid, bx, 0, s>>>(P, st, phi0, cA0, cB0);
     }
+    // ``in_step``: the first kernel of a step (see begin_after_previous); the diagnostics' phi pass
+    // stands between kernels launched the plain way and is cheaper to queue like them
     template <int LAT>
-    static void phi(const DevParams& P, const StateView& st, int mode, void* phi_work, cudaStream_t s) {
-        int bx; const dim3 grid = node_grid(P, bx);
+    static void phi(const DevParams& P, const StateView& st, int mode, void* phi_work, cudaStream_t s,
+                    bool in_step = false) {
+        int bx; const dim3 grid = step_grid(P, bx);
         R* ph = static_cast<R*>(phi_work);
-        LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M><<<grid, bx, 0, s>>>(P, st, ph));
+        if (in_step) {
+            LBM_MODE_SWITCH(mode, launch_after_previous<R>(phi_kernel<T, LAT, M>, grid, dim3(bx), 0, s, P, st, ph));
+        } else {
+            LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M><<<grid, bx, 0, s>>>(P, st, ph));
+        }
     }
     template <int LAT>
     static void plane_phi(const DevParams& P, const StateView& st, int mode, int z, void* out, cudaStream_t s) {
@@ -1293,16 +1342,16 @@ struct Launchers {
     template <int LAT, bool FLOW>
     static void step(const DevParams& P, const StateView& st, const StateView& out, int mode, void* phi_work,
                      cudaStream_t s) {
-        int bx; const dim3 grid = node_grid(P, bx);
+        int bx; const dim3 grid = step_grid(P, bx);
         R* phi = static_cast<R*>(phi_work);
         // MRT in an instance of its own: its 19 x 19 transform would raise every instance's registers
         if constexpr (FLOW) {
             if (P.coll == 2) {
-                LBM_MODE_SWITCH(mode, step_kernel<T, LAT, FLOW, M, 2><<<grid, bx, 0, s>>>(P, st, out, phi));
+                LBM_MODE_SWITCH(mode, launch_after_previous<R>(step_kernel<T, LAT, FLOW, M, 2>, grid, dim3(bx), 0, s, P, st, out, phi));
                 return;
             }
         }
-        LBM_MODE_SWITCH(mode, step_kernel<T, LAT, FLOW, M, -1><<<grid, bx, 0, s>>>(P, st, out, phi));
+        LBM_MODE_SWITCH(mode, launch_after_previous<R>(step_kernel<T, LAT, FLOW, M, -1>, grid, dim3(bx), 0, s, P, st, out, phi));
     }
     static void fused(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
         const dim3 block(FX, FY);
@@ -1339,15 +1388,15 @@ struct Launchers {
             configured |= 1ull << dev;
         }
         const bool slab = P.z_lo != 0 || P.z_hi != P.nz || P.wall_zlo != P.wall_z || P.wall_zhi != P.wall_z;
-        if (slab) fused_flow_kernel<T, COLL, true><<<grid, block, smem, s>>>(P, src, dst, zchunk);
-        else fused_flow_kernel<T, COLL, false><<<grid, block, smem, s>>>(P, src, dst, zchunk);
+        if (slab) launch_after_previous<R>(fused_flow_kernel<T, COLL, true>, grid, block, smem, s, P, src, dst, zchunk);
+        else launch_after_previous<R>(fused_flow_kernel<T, COLL, false>, grid, block, smem, s, P, src, dst, zchunk);
     }
     template <int LAT, bool FLOW>
     static void fields(const DevParams& P, const StateView& st, int mode, void* phi_work, FieldPtrs out,
                        cudaStream_t s) {
         int bx; const dim3 grid = node_grid(P, bx);
         R* phi = static_cast<R*>(phi_work);
-        if constexpr (FLOW) { LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M><<<grid, bx, 0, s>>>(P, st, phi)); }
+        if constexpr (FLOW) Launchers::template phi<LAT>(P, st, mode, phi_work, s);
         LBM_MODE_SWITCH(mode, fields_kernel<T, LAT, FLOW, M><<<grid, bx, 0, s>>>(P, st, phi, out));
     }
     // Blocks of 256 threads of ``kernel`` that the device holds at once, at most ``cap``: a
@@ -1372,8 +1421,7 @@ struct Launchers {
         R* phi = static_cast<R*>(phi_work);
         unsigned* bits = static_cast<unsigned*>(bits_work);
         if constexpr (FLOW || kTwoD<LAT>) {
-            int bx; const dim3 grid = node_grid(P, bx);
-            LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M><<<grid, bx, 0, s>>>(P, st, phi));
+            Launchers::template phi<LAT>(P, st, mode, phi_work, s);
         }
         int nb = nblocks;
         LBM_MODE_SWITCH(mode, {
@@ -1403,10 +1451,10 @@ struct Launchers {
     }                                                                                                     \
     void launch_phi_##SUFFIX(const DevParams& P, const StateView& st, int lat, int mode, void* phi,       \
                              cudaStream_t s) {                                                            \
-        if (lat == LAT_D2Q5) Launchers<T>::phi<LAT_D2Q5>(P, st, mode, phi, s);                             \
-        else if (lat == LAT_D2Q9) Launchers<T>::phi<LAT_D2Q9>(P, st, mode, phi, s);                        \
-        else if (lat == LAT_D3Q19) Launchers<T>::phi<LAT_D3Q19>(P, st, mode, phi, s);                      \
-        else Launchers<T>::phi<LAT_D3Q7>(P, st, mode, phi, s);                                             \
+        if (lat == LAT_D2Q5) Launchers<T>::phi<LAT_D2Q5>(P, st, mode, phi, s, true);                             \
+        else if (lat == LAT_D2Q9) Launchers<T>::phi<LAT_D2Q9>(P, st, mode, phi, s, true);                        \
+        else if (lat == LAT_D3Q19) Launchers<T>::phi<LAT_D3Q19>(P, st, mode, phi, s, true);                      \
+        else Launchers<T>::phi<LAT_D3Q7>(P, st, mode, phi, s, true);                                             \
     }                                                                                                     \
     void launch_plane_phi_##SUFFIX(const DevParams& P, const StateView& st, int lat, int mode, int z,    \
                                    void* out, cudaStream_t s) {                                           \
