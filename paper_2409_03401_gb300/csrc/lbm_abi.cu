@@ -274,15 +274,18 @@ int read_mode(const lbm_ctx* c) {
     return (c->t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven;
 }
 // Whether a flow step of the two-buffer layout runs as the fused kernel: FP32 storage from
-// 600,000 nodes on, and slabs (whose ghost phi it reads in place). The others take a phi pass and
-// the per-node pull step, the same fields bit for bit. The fused kernel computes phi of its halo
-// again (a third more): that saves HBM traffic, but 16-bit and FP64 storage pay for it in issue
-// slots and on the FP64 pipe (512^3 FP16 8.01 ms against 7.29 for the two passes, 64^3 27 against
-// 21 us; FP64 128^3 2.45 against 2.16 ms), and in lattices that stay in L2 its planes, one after
-// another, take longer than two launches (FP32 64^3 24 against 18 us, 80^3 44 against 43 us,
-// 96^3 61 against 68 us).
+// 600,000 nodes on, BF16 storage, and slabs (whose ghost phi it reads in place). The others take
+// a phi pass and the per-node pull step, the same fields bit for bit. The fused kernel computes
+// phi of its halo again (a third more): that saves HBM traffic, but FP16 and FP64 storage pay
+// for it in issue slots and on the FP64 pipe (512^3 FP16 8.01 ms against 7.29 for the two
+// passes, 64^3 27 against 21 us; FP64 128^3 2.45 against 2.16 ms), and in lattices that stay in
+// L2 its planes, one after another, take longer than two launches (FP32 64^3 24 against 18 us,
+// 80^3 44 against 43 us, 96^3 61 against 68 us). BF16 would gain as FP16 does, but the compiler
+// fuses other multiply-adds of its flow collision in the two kernels, and an 8-bit significand
+// turns that into fields 1e-3 apart after 30 steps.
 bool one_pass(const lbm_ctx* c) {
-    return c->L.two && fused_flow(&c->p) && (c->slab || (c->p.storage == LBM_F32 && c->L.n >= 600000));
+    if (!c->L.two || !fused_flow(&c->p)) return false;
+    return c->slab || c->p.storage == LBM_BF16 || (c->p.storage == LBM_F32 && c->L.n >= 600000);
 }
 
 }  // namespace
