@@ -165,6 +165,16 @@ lbm_status lbm_attach(const lbm_params* p, void* d_state, void* d_work, int64_t 
  * the capillary stencil (lbm_kernels_per_step). Asynchronous. */
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
 
+/* lbm_step with a scratch buffer: with FP32 storage and no flow (LBM_D3Q7 from a million nodes
+ * on, LBM_D2Q5, and LBM_D2Q9 without x walls) every four steps from an even time level are two passes over
+ * memory, from the state to the scratch buffer and back, with two steps in each. Same results
+ * as lbm_step, bit for bit. lbm_step_scratch_bytes is the size wanted (one state copy; 0 where
+ * it does not apply). d_scratch: 256-byte aligned device memory of the caller's, used only by
+ * the work this call queues; NULL or fewer bytes take lbm_step's path, as do steps recorded by
+ * lbm_profile_begin and slabs. Asynchronous. No counterpart in the paper. */
+size_t lbm_step_scratch_bytes(const lbm_params* p);
+lbm_status lbm_step_scratch(lbm_ctx* ctx, int nsteps, void* d_scratch, size_t scratch_bytes);
+
 /* Advance nsteps coupled time steps by replaying a CUDA graph of two steps (captured on the
  * first call from an even time level, after one plain pair of steps; kept until
  * lbm_destroy): the same kernels and results as lbm_step, bit for bit, with one launch per

@@ -404,6 +404,76 @@ __device__ __forceinline__ void mrt_relax(const DevParams& P, Pre d_of, Post put
     }
 }
 
+// Collisions of g, h^A, h^B at a node at rest (no flow: every e.u term of Eqs. 47 and 51 is 0
+// and left out). ``emit(set, k, r)`` takes the post-collision population k > 0 of set SET_G
+// (g), SET_H (h^A) or SET_H + 1 (h^B) in storage units and returns it as stored; the rest
+// populations, in natural units, follow as emit(set, 0, r).
+template <class T, int LAT, class Emit>
+__device__ __forceinline__ void collide_at_rest(const Node<T, LAT, false>& nd, const DevParams& P, Emit emit) {
+    using R = typename RealOf<T>::type;
+    using L = Scalar<LAT>;
+    constexpr int Q = L::Q;
+    const R phi = nd.phi();
+    const R p = interp_p(phi);
+    const R muA = closure_dev(nd.dcA, p, 0, P);
+    const R muB = closure_dev(nd.dcB, p, 1, P);
+    const R inv_cs2 = R(1.0 / L::cs2());
+    const R omg = coef<R>(P).om_g;
+    const R MA = coef<R>(P).M0[0] * (R(1) - phi) + coef<R>(P).M1[0] * phi;     // §2.3
+    const R MB = coef<R>(P).M0[1] * (R(1) - phi) + coef<R>(P).M1[1] * phi;
+    const R omA = recip(MA * inv_cs2 + R(0.5));                      // tau_h = M / c_s^2
+    const R omB = recip(MB * inv_cs2 + R(0.5));
+    const R ga = phi - R(0.5) * nd.S;
+    // rest populations: the conserved totals minus the moving populations (see collide_store)
+    R g0, hA0 = nd.dcA, hB0 = nd.dcB;
+    if constexpr (!is16<T>()) {
+        g0 = phi + R(0.5) * nd.S;                                     // phi~ + S
+#pragma unroll
+        for (int k = 1; k < Q; ++k) {
+            const R w = R(L::w(k));
+            g0 -= emit(int(SET_G), k, nd.g[k] - omg * (nd.g[k] - w * ga) + w * nd.S);
+            hA0 -= emit(int(SET_H), k, nd.hA[k] - omA * (nd.hA[k] - w * muA));
+            hB0 -= emit(int(SET_H) + 1, k, nd.hB[k] - omB * (nd.hB[k] - w * muB));
+        }
+    } else {
+        using C = Codec<T>;
+        constexpr float uh = C::template unit<SET_H>();
+        g0 = phi + R(0.5) * nd.S - R(0.5 * (1.0 - L::w(0)));
+        const R gq = R(0.5) - ga;
+        const R mA = R(uh) * muA, mB = R(uh) * muB;
+#pragma unroll
+        for (int k = 1; k < Q; ++k) {
+            g0 -= R(C::template scale<SET_G>(L::w(k))) * emit(int(SET_G), k, nd.g[k] - omg * (nd.g[k] + gq) + nd.S);
+            hA0 -= R(C::template scale<SET_H>(L::w(k))) * emit(int(SET_H), k, nd.hA[k] - omA * (nd.hA[k] - mA));
+            hB0 -= R(C::template scale<SET_H>(L::w(k))) * emit(int(SET_H) + 1, k, nd.hB[k] - omB * (nd.hB[k] - mB));
+        }
+    }
+    emit(int(SET_G), 0, g0);
+    emit(int(SET_H), 0, hA0);
+    emit(int(SET_H) + 1, 0, hB0);
+}
+
+// Store population k of set ``set`` (see collide_at_rest) to slot s; returns it as stored.
+template <class T, int LAT>
+__device__ __forceinline__ typename RealOf<T>::type store_at(const StateView& st, int set, int k, Slot s,
+                                                             typename RealOf<T>::type r) {
+    using PL = Planes<LAT>;
+    T* e = set == SET_G ? element<T, PL::G>(st, k, s)
+         : (set == SET_H ? element<T, PL::HA>(st, k, s) : element<T, PL::HB>(st, k, s));
+    if constexpr (is16<T>()) {
+        return set == SET_G ? Codec<T>::template store_back<SET_G>(e, r) : Codec<T>::template store_back<SET_H>(e, r);
+    } else {
+        *e = r;
+        return r;
+    }
+}
+template <class T, int LAT>
+__device__ __forceinline__ void store_rest_at(const StateView& st, int set, int node, typename RealOf<T>::type r,
+                                              const DevParams& P) {
+    if constexpr (is16<T>()) st.rest[(set - SET_G) * P.plane + node] = float(r);
+    else store_at<T, LAT>(st, set, 0, Slot{node, 0}, r);
+}
+
 template <class T, int LAT, bool FLOW, class A, int COLL = -2>
 __device__ __forceinline__ void collide_store(const Node<T, LAT, FLOW>& nd, typename RealOf<T>::type phi,
                                               typename RealOf<T>::type ux, typename RealOf<T>::type uy,
@@ -674,15 +744,18 @@ step_kernel(const DevParams P, const StateView st, const StateView out,
     Node<T, LAT, FLOW> nd;
     nd.gather(st, ad, P);
     nd.moments(P);
-    R phi;
-    if constexpr (FLOW) phi = phi_field[ad.self]; else phi = nd.phi();
-    R ux = R(0), uy = R(0), uz = R(0), Fx = R(0), Fy = R(0), Fz = R(0);
     if constexpr (FLOW) {
-        R gx, gy, gz, lap;
+        const R phi = phi_field[ad.self];
+        R ux, uy, uz, Fx, Fy, Fz, gx, gy, gz, lap;
         stencil([&](int dx, int dy, int dz) { return ad.phi(phi_field, dx, dy, dz); }, phi, gx, gy, gz, lap);
         force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
+        collide_store<T, LAT, FLOW, Addr<MODE>, COLL>(nd, phi, ux, uy, uz, Fx, Fy, Fz, out, ad, P);
+    } else {
+        collide_at_rest<T, LAT>(nd, P, [&](int set, int k, R r) {
+            if (k == 0) { store_rest_at<T, LAT>(out, set, ad.self, r, P); return r; }
+            return store_at<T, LAT>(out, set, k, ad.dst(k, Scalar<LAT>::ex(k), Scalar<LAT>::ey(k), Scalar<LAT>::ez(k)), r);
+        });
     }
-    collide_store<T, LAT, FLOW, Addr<MODE>, COLL>(nd, phi, ux, uy, uz, Fx, Fy, Fz, out, ad, P);
 }
 
 // phi = sum g + S/2 of every node (Eq. 49), read by the capillary stencil.
@@ -1279,6 +1352,12 @@ inline int march_chunk(long long tiles, int n, long long slots, double extra) {
     return best;
 }
 
+}  // namespace lbm
+
+#include "lbm_two_steps.cuh"
+
+namespace lbm {
+
 // ------------------------------------------------------------------------------------
 // Host launchers for one storage type. ``mode`` is AA_EVEN / AA_ODD for the in-place
 // layout and PULL for the two-buffer layout (st = the current state buffer).
@@ -1352,6 +1431,10 @@ struct Launchers {
             }
         }
         LBM_MODE_SWITCH(mode, launch_after_previous<R>(step_kernel<T, LAT, FLOW, M, -1>, grid, dim3(bx), 0, s, P, st, out, phi));
+    }
+    template <int LAT>
+    static void two_steps(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
+        launch_two_steps_at<T, LAT>(P, src, dst, s);
     }
     static void fused(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
         const dim3 block(FX, FY);
@@ -1471,6 +1554,14 @@ struct Launchers {
         else if (lat == LAT_D3Q19) Launchers<T>::step<LAT_D3Q19, false>(P, st, out, mode, phi, s);         \
         else if (flow) Launchers<T>::step<LAT_D3Q7, true>(P, st, out, mode, phi, s);                       \
         else Launchers<T>::step<LAT_D3Q7, false>(P, st, out, mode, phi, s);                                \
+    }                                                                                                     \
+    void launch_two_steps_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst, int lat, \
+                                   cudaStream_t s) {                                                      \
+        if constexpr (sizeof(T) == 4) {                                                                   \
+            if (lat == LAT_D2Q5) Launchers<T>::two_steps<LAT_D2Q5>(P, src, dst, s);                        \
+            else if (lat == LAT_D2Q9) Launchers<T>::two_steps<LAT_D2Q9>(P, src, dst, s);                   \
+            else Launchers<T>::two_steps<LAT_D3Q7>(P, src, dst, s);                                       \
+        }                                                                                                 \
     }                                                                                                     \
     void launch_fused_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst,            \
                                cudaStream_t s) {                                                          \

@@ -25,6 +25,8 @@ constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
                                    cudaStream_t);                                                        \
     void launch_step_##SUFFIX(const DevParams&, const StateView&, const StateView&, int lat, bool flow, \
                               int mode, void* phi, cudaStream_t);                                        \
+    void launch_two_steps_##SUFFIX(const DevParams&, const StateView&, const StateView&, int lat,        \
+                                   cudaStream_t);                                                         \
     void launch_fused_##SUFFIX(const DevParams&, const StateView&, const StateView&, cudaStream_t);       \
     void launch_fields_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, int mode,        \
                                 void* phi, FieldPtrs, cudaStream_t);                                     \

@@ -127,9 +127,33 @@ class Simulation:
     def step(self, n=1, graph=False):
         """Advance n steps; ``graph=True`` replays a captured CUDA graph of two steps (needs a
         created stream, e.g. Simulation(..., stream=torch.cuda.Stream()))."""
+        scratch = None if graph or n < 4 else self._scratch()
+        if scratch is not None:
+            _lib.check(self.lib.lbm_step_scratch(self._ctx, int(n), _ptr(scratch), scratch.numel()), self._ctx)
+            return self
         fn = self.lib.lbm_step_graph if graph else self.lib.lbm_step
         _lib.check(fn(self._ctx, int(n)), self._ctx)
         return self
+
+    def _scratch(self):
+        """One state copy from torch's allocator for lbm_step_scratch, on the simulation's stream
+        (returned to the allocator after the call, which reuses it in stream order), or None
+        where the library takes no scratch, while the stream is being captured, for a copy above
+        an eighth of the device's memory, or when the memory is not there."""
+        if not hasattr(self, "_scratch_bytes"):
+            b = self.lib.lbm_step_scratch_bytes(ctypes.byref(self._cp))
+            if b and b > torch.cuda.get_device_properties(self.device).total_memory // 8:
+                b = 0
+            self._scratch_bytes = b
+        if not self._scratch_bytes:
+            return None
+        with torch.cuda.stream(self.stream):
+            if torch.cuda.is_current_stream_capturing():
+                return None
+            try:
+                return torch.empty(self._scratch_bytes, dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                return None
 
     def fields(self, names=_lib.FIELDS):
         """Dict of (nz, ny, nx) tensors of the current time level."""

@@ -52,3 +52,68 @@ def _compare_with_fused(p, steps):
         _lib.check(lib.lbm_step_buffers(ctypes.byref(cp), at[t % 2], at[1 - t % 2], t, None,
                                         ctypes.c_void_p(b.stream.cuda_stream)))
     _same(a.fields(), Simulation.attach(p, b.state, steps).fields())
+
+
+def _two_against_single(p, steps=(8, 1, 9, 7, 4)):
+    # two steps per pass (the scratch buffer lent here whatever the lattice's size) and single steps
+    from paper_2409_03401_gb300 import Simulation, _lib
+    lib = _lib.load()
+    f = _inputs(p)
+    a, b = (Simulation(p, *f, device="cuda") for _ in range(2))
+    scratch = torch.empty(lib.lbm_copy_bytes(ctypes.byref(a._cp)), dtype=torch.uint8, device="cuda")
+    for n in steps:
+        _lib.check(lib.lbm_step_scratch(a._ctx, n, ctypes.c_void_p(scratch.data_ptr()), scratch.numel()), a._ctx)
+        _lib.check(lib.lbm_step(b._ctx, n), b._ctx)
+        assert a.t == b.t
+        _same(a.fields(), b.fields())
+
+
+@pytest.mark.parametrize("wall_x,wall_z", [(False, False), (True, False), (False, True), (True, True)])
+def test_two_steps_per_pass_match_single_steps_3d(wall_x, wall_z):
+    # 1,008,000 nodes, just over the size rule: several 28 x 14 tiles with ragged ends
+    _two_against_single(LBMParams(150, 84, 80, wall_x=wall_x, wall_z=wall_z), (8, 1, 7))
+
+
+@pytest.mark.parametrize("nx", [1, 2, 27, 28, 29, 57, 512])
+@pytest.mark.parametrize("ny", [1, 3, 90])
+def test_two_steps_per_pass_match_single_steps_2d(nx, ny):
+    # window edges (28 nodes), lattices narrower than a window, one-row lattices, walls in x
+    _two_against_single(LBMParams(nx, ny, 1, lattice="D2Q9"))
+    _two_against_single(LBMParams(nx, ny, 1, lattice="D2Q5"))
+    _two_against_single(LBMParams(nx, ny, 1, lattice="D2Q5", wall_x=True))
+
+
+def test_step_scratch_takes_what_it_can_use_and_no_more():
+    from paper_2409_03401_gb300 import LBMError, Simulation, _lib
+    lib = _lib.load()
+    p = LBMParams(128, 96, 96)
+    f = _inputs(p)
+    a, b = (Simulation(p, *f, device="cuda") for _ in range(2))
+    need = lib.lbm_step_scratch_bytes(ctypes.byref(a._cp))
+    assert need == lib.lbm_copy_bytes(ctypes.byref(a._cp)) > 0
+    for q in (p.with_(flow=True), p.with_(storage="f64"), p.with_(storage="f16"), p.with_(lattice="D3Q19"),
+              p.with_(nx=32), LBMParams(64, 64, 1, lattice="D2Q9", wall_x=True)):
+        assert lib.lbm_step_scratch_bytes(ctypes.byref(_lib.make_params(q))) == 0
+    guard = 1 << 16
+    buf = torch.full((need + 2 * guard,), 0xA5, dtype=torch.uint8, device="cuda")
+    with pytest.raises(LBMError):
+        _lib.check(lib.lbm_step_scratch(a._ctx, 4, ctypes.c_void_p(buf.data_ptr() + 8), need), a._ctx)
+    assert a.t == 0
+    short = ctypes.c_void_p(buf.data_ptr() + guard)
+    _lib.check(lib.lbm_step_scratch(a._ctx, 5, short, need - 1), a._ctx)         # too small: single steps
+    assert bool((buf == 0xA5).all())
+    _lib.check(lib.lbm_step_scratch(a._ctx, 6, short, need), a._ctx)
+    b.step(3).step(8)
+    _same(a.fields(), b.fields())
+    assert bool((buf[:guard] == 0xA5).all()) and bool((buf[guard + need:] == 0xA5).all())
+    # a stream under capture takes the single steps, and the graph replays them
+    s = torch.cuda.Stream()
+    c = Simulation(p, *f, device="cuda", stream=s)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        c.step(6)
+    g.replay()
+    torch.cuda.synchronize()
+    d = Simulation(p, *f, device="cuda").step(6)
+    _same(c.fields(), d.fields())
