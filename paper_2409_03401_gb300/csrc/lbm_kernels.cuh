@@ -149,6 +149,36 @@ struct AddrInterior {
     __device__ __forceinline__ Slot dst(int k, int, int, int) const { return {self, k}; }
 };
 
+// Addr<MODE> at a node whose neighbours all lie inside the lattice: no wrap and no wall, so
+// every slot is at an offset from the node that is the same for the whole block.
+template <int MODE>
+struct AddrInner {
+    static constexpr int kF0In = Addr<MODE>::kF0In, kF0Out = Addr<MODE>::kF0Out;
+    int self;
+    int sx, sxy;   // nx, nx * ny
+    __device__ __forceinline__ int beside(int ex, int ey, int ez) const { return self + ex + ey * sx + ez * sxy; }
+    __device__ __forceinline__ Slot src(int k, int ex, int ey, int ez) const {
+        if (MODE == AA_EVEN || k == 0) return {self, k};
+        return {beside(-ex, -ey, -ez), MODE == AA_ODD ? opp(k) : k};
+    }
+    __device__ __forceinline__ Slot dst(int k, int ex, int ey, int ez) const {
+        if (k == 0 || MODE == PULL) return {self, k};
+        return MODE == AA_EVEN ? Slot{self, opp(k)} : Slot{beside(ex, ey, ez), k};
+    }
+    __device__ __forceinline__ int writer(int k, int ex, int ey, int ez) const {
+        return k == 0 ? self : beside(-ex, -ey, -ez);
+    }
+    template <class R>
+    __device__ __forceinline__ R phi(const R* __restrict__ f, int dx, int dy, int dz) const {
+        return f[beside(dx, dy, dz)];
+    }
+};
+// Whether the 32 nodes of this thread's warp (x of its first lane, row y, plane z) are such nodes.
+__device__ __forceinline__ bool warp_inside(int x, int y, int z, const DevParams& P) {
+    const int x0 = x - int(threadIdx.x & 31);
+    return x0 >= 1 && x0 + 32 < P.nx && y >= 1 && y + 1 < P.ny && z >= 1 && z + 1 < P.nz;
+}
+
 // Incoming populations of one node and their moments (steps a1-a3 of one node).
 // The rest populations h_0 are stored shifted by c_0^eq (a constant shift commutes with
 // the BGK relaxation of Eq. 50), so sum_k h_k gives dc = c - c_0^eq without the
@@ -726,6 +756,28 @@ __device__ __forceinline__ void collide_store(const Node<T, LAT, FLOW>& nd, type
     }
 }
 
+// The step of one node at address ``ad``.
+template <class T, int LAT, bool FLOW, int COLL, class A>
+__device__ __forceinline__ void step_node(const A& ad, const DevParams& P, const StateView& st, const StateView& out,
+                                          const typename RealOf<T>::type* __restrict__ phi_field) {
+    using R = typename RealOf<T>::type;
+    Node<T, LAT, FLOW> nd;
+    nd.gather(st, ad, P);
+    nd.moments(P);
+    if constexpr (FLOW) {
+        const R phi = phi_field[ad.self];
+        R ux, uy, uz, Fx, Fy, Fz, gx, gy, gz, lap;
+        stencil([&](int dx, int dy, int dz) { return ad.phi(phi_field, dx, dy, dz); }, phi, gx, gy, gz, lap);
+        force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
+        collide_store<T, LAT, FLOW, A, COLL>(nd, phi, ux, uy, uz, Fx, Fy, Fz, out, ad, P);
+    } else {
+        collide_at_rest<T, LAT>(nd, P, [&](int set, int k, R r) {
+            if (k == 0) { store_rest_at<T, LAT>(out, set, ad.self, r, P); return r; }
+            return store_at<T, LAT>(out, set, k, ad.dst(k, Scalar<LAT>::ex(k), Scalar<LAT>::ey(k), Scalar<LAT>::ez(k)), r);
+        });
+    }
+}
+
 // ------------------------------------------------------------------------------------
 // One coupled step per node. With flow the phi field of this step must already be in
 // phi_field (phi pass); MODE AA_* works in place on ``st``, PULL reads ``st`` and writes ``out``.
@@ -738,24 +790,19 @@ step_kernel(const DevParams P, const StateView st, const StateView out,
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
+    // warps inside the lattice skip the wrap tests where that measured faster (256^3 in place: even
+    // FP32 steps 1016 -> 914 us, odd 16-bit ones 894 -> 869 us; elsewhere the extra registers of
+    // the second path cost more than it saves, e.g. the FP16 pull step 739 -> 768 us)
+    if constexpr (FLOW && (is16<T>() ? MODE == AA_ODD : MODE == AA_EVEN)) {
+        if (warp_inside(x, y, z, P)) {
+            step_node<T, LAT, FLOW, COLL>(AddrInner<MODE>{node_of(x, y, z, P), P.nx, P.nx * P.ny}, P, st, out, phi_field);
+            return;
+        }
+    }
     Addr<MODE> ad;
     ad.self = node_of(x, y, z, P);
     ad.nb.init(x, y, z, P);
-    Node<T, LAT, FLOW> nd;
-    nd.gather(st, ad, P);
-    nd.moments(P);
-    if constexpr (FLOW) {
-        const R phi = phi_field[ad.self];
-        R ux, uy, uz, Fx, Fy, Fz, gx, gy, gz, lap;
-        stencil([&](int dx, int dy, int dz) { return ad.phi(phi_field, dx, dy, dz); }, phi, gx, gy, gz, lap);
-        force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
-        collide_store<T, LAT, FLOW, Addr<MODE>, COLL>(nd, phi, ux, uy, uz, Fx, Fy, Fz, out, ad, P);
-    } else {
-        collide_at_rest<T, LAT>(nd, P, [&](int set, int k, R r) {
-            if (k == 0) { store_rest_at<T, LAT>(out, set, ad.self, r, P); return r; }
-            return store_at<T, LAT>(out, set, k, ad.dst(k, Scalar<LAT>::ex(k), Scalar<LAT>::ey(k), Scalar<LAT>::ez(k)), r);
-        });
-    }
+    step_node<T, LAT, FLOW, COLL>(ad, P, st, out, phi_field);
 }
 
 // phi = sum g + S/2 of every node (Eq. 49), read by the capillary stencil.
@@ -766,13 +813,22 @@ phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* __re
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
+    auto phi_at = [&](const auto& ad) {
+        Node<T, LAT, false> nd;
+        nd.gather_scalars(st, ad, P);
+        nd.moments(P);
+        phi_out[ad.self] = nd.phi();
+    };
+    if constexpr (LAT == LAT_D3Q19) {       // 57 gathers: FP32 600 -> 574 us at 256^3, FP16 556 -> 457 us
+        if (warp_inside(x, y, z, P)) {
+            phi_at(AddrInner<MODE>{node_of(x, y, z, P), P.nx, P.nx * P.ny});
+            return;
+        }
+    }
     Addr<MODE> ad;
     ad.self = node_of(x, y, z, P);
     ad.nb.init(x, y, z, P);
-    Node<T, LAT, false> nd;
-    nd.gather_scalars(st, ad, P);
-    nd.moments(P);
-    phi_out[ad.self] = nd.phi();
+    phi_at(ad);
 }
 
 // phi (Eq. 49) of plane z into out[y nx + x]: a slab's edge plane, sent to the neighbouring
