@@ -791,9 +791,10 @@ step_kernel(const DevParams P, const StateView st, const StateView out,
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
     // warps inside the lattice skip the wrap tests where that measured faster (256^3 in place: even
-    // FP32 steps 1016 -> 914 us, odd 16-bit ones 894 -> 869 us; elsewhere the extra registers of
-    // the second path cost more than it saves, e.g. the FP16 pull step 739 -> 768 us)
-    if constexpr (FLOW && (is16<T>() ? MODE == AA_ODD : MODE == AA_EVEN)) {
+    // FP32 steps 1016 -> 914 us; odd and pull steps lose more to the extra registers of the second
+    // path). 16-bit storage keeps one path: a multiply-add fused otherwise in a second one would
+    // round some populations to the next 16-bit value.
+    if constexpr (FLOW && !is16<T>() && MODE == AA_EVEN) {
         if (warp_inside(x, y, z, P)) {
             step_node<T, LAT, FLOW, COLL>(AddrInner<MODE>{node_of(x, y, z, P), P.nx, P.nx * P.ny}, P, st, out, phi_field);
             return;
@@ -819,7 +820,7 @@ phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* __re
         nd.moments(P);
         phi_out[ad.self] = nd.phi();
     };
-    if constexpr (LAT == LAT_D3Q19) {       // 57 gathers: FP32 600 -> 574 us at 256^3, FP16 556 -> 457 us
+    if constexpr (LAT == LAT_D3Q19 && !is16<T>()) {       // 57 gathers: FP32 600 -> 574 us at 256^3
         if (warp_inside(x, y, z, P)) {
             phi_at(AddrInner<MODE>{node_of(x, y, z, P), P.nx, P.nx * P.ny});
             return;
