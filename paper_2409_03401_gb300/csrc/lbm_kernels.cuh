@@ -1202,6 +1202,17 @@ __device__ __forceinline__ int euler_quads4(const R* __restrict__ phi, int x, in
 // node it bounds is set (b[c][b][a]: node (x - 1 + a, y - 1 + b, z - 1 + c)). Outside an x
 // or z wall is empty; other axes wrap. bits: bit (id & 31) of word id >> 5 is node id's
 // phi >= 1/2, ids x fastest.
+__device__ __forceinline__ int euler_of_cells(const int (&b)[2][2][2]) {
+    const int vert = b[0][0][0] | b[0][0][1] | b[0][1][0] | b[0][1][1] | b[1][0][0] | b[1][0][1] | b[1][1][0] |
+                     b[1][1][1];
+    const int ex = b[0][0][1] | b[0][1][1] | b[1][0][1] | b[1][1][1];
+    const int ey = b[0][1][0] | b[0][1][1] | b[1][1][0] | b[1][1][1];
+    const int ez = b[1][0][0] | b[1][0][1] | b[1][1][0] | b[1][1][1];
+    const int fx = b[1][1][0] | b[1][1][1];
+    const int fy = b[1][0][1] | b[1][1][1];
+    const int fz = b[0][1][1] | b[1][1][1];
+    return vert - (ex + ey + ez) + (fx + fy + fz) - b[1][1][1];
+}
 __device__ __forceinline__ int euler_cells(const unsigned* __restrict__ bits, int x, int y, int z,
                                            const DevParams& P) {
     int b[2][2][2];
@@ -1221,15 +1232,7 @@ __device__ __forceinline__ int euler_cells(const unsigned* __restrict__ bits, in
                 const unsigned id = (unsigned(zz) * unsigned(P.ny) + unsigned(yy)) * unsigned(P.nx) + unsigned(xx);
                 b[c][bb][a] = inside ? int((__ldg(bits + (id >> 5)) >> (id & 31)) & 1u) : 0;
             }
-    const int vert = b[0][0][0] | b[0][0][1] | b[0][1][0] | b[0][1][1] | b[1][0][0] | b[1][0][1] | b[1][1][0] |
-                     b[1][1][1];
-    const int ex = b[0][0][1] | b[0][1][1] | b[1][0][1] | b[1][1][1];
-    const int ey = b[0][1][0] | b[0][1][1] | b[1][1][0] | b[1][1][1];
-    const int ez = b[1][0][0] | b[1][0][1] | b[1][1][0] | b[1][1][1];
-    const int fx = b[1][1][0] | b[1][1][1];
-    const int fy = b[1][0][1] | b[1][1][1];
-    const int fz = b[0][1][1] | b[1][1][1];
-    return vert - (ex + ey + ez) + (fx + fy + fz) - b[1][1][1];
+    return euler_of_cells(b);
 }
 
 // Writes slot LBM_RED_EULER of every block's partials (the reduction kernel leaves it 0 on
@@ -1300,16 +1303,76 @@ template <class T, int LAT> constexpr int reduce_min_blocks() {
     return (LAT == LAT_D3Q19 || sizeof(typename RealOf<T>::type) == 8) ? 2 : 3;
 }
 
+// Running sums of one thread over the nodes it visits.
+template <class R>
+struct NodeSums {
+    SumAcc<R> phi, dcA, dcB, p, S, phit, interface;
+    R umax = R(0);
+    int nodes = 0, bad = 0;
+    __device__ __forceinline__ void add(R ph, R a, R b, R pr, R s, R pt, R umag, R kint) {
+        phi.add(ph);
+        dcA.add(a);
+        dcB.add(b);
+        p.add(pr);
+        S.add(s);
+        phit.add(pt);
+        interface.add(kint * ph * (R(1) - ph));                        // Eq. 67 integrand
+        ++nodes;
+        const bool finite = isfinite(ph) && isfinite(a) && isfinite(b) && isfinite(pr) && isfinite(s) &&
+                            isfinite(umag) && isfinite(pt);
+        bad += finite ? 0 : 1;
+        if (isfinite(umag)) umax = umag > umax ? umag : umax;
+    }
+    // block totals into row ``row`` of the partials; the whole block calls it (256 threads)
+    __device__ __forceinline__ void write(double euler, int tid, long long row, const DevParams& P,
+                                          double* __restrict__ partials) const {
+        double acc[LBM_NRED_DEV];
+        acc[0] = phi.value();
+        acc[1] = dcA.value() + double(nodes) * P.c0[0];
+        acc[2] = dcB.value() + double(nodes) * P.c0[1];
+        acc[3] = p.value();
+        acc[4] = S.value();
+        acc[5] = double(umax);
+        acc[6] = phit.value();
+        acc[7] = double(bad);
+        acc[8] = interface.value();
+        acc[9] = euler;
+        // warp shuffles, then one warp over the warp results
+        __shared__ double sm[LBM_NRED_DEV][32];
+        const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+        for (int i = 0; i < LBM_NRED_DEV; ++i) {
+            double v = acc[i];
+            for (int o = 16; o > 0; o >>= 1) {
+                const double u = __shfl_down_sync(0xffffffffu, v, o);
+                v = (i == 5) ? fmax(v, u) : v + u;
+            }
+            if (lane == 0) sm[i][warp] = v;
+        }
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int i = 0; i < LBM_NRED_DEV; ++i) {
+                double v = lane < 8 ? sm[i][lane] : 0.0;
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double u = __shfl_down_sync(0xffffffffu, v, o);
+                    v = (i == 5) ? fmax(v, u) : v + u;
+                }
+                if (lane == 0) partials[row * LBM_NRED_DEV + i] = v;
+            }
+        }
+    }
+};
+
 template <class T, int LAT, bool FLOW, int MODE>
 __global__ void __launch_bounds__(256, (reduce_min_blocks<T, LAT>()))
 reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::type* __restrict__ phi_field,
               unsigned* __restrict__ bits, double* __restrict__ partials) {
     using R = typename RealOf<T>::type;
-    SumAcc<R> s_phi, s_dcA, s_dcB, s_p, s_S, s_phit, s_int;
-    R umax = R(0);
-    int nodes = 0, bad = 0, quads = 0;
+    NodeSums<R> sums;
+    int quads = 0;
     const R kint = R(4.0 / P.W);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const unsigned nxy = unsigned(P.nx) * unsigned(P.ny);
     const unsigned stride = gridDim.x * blockDim.x;
     // nodes of the planes [z_lo, z_hi); the bit field (3D Euler count) only when they start at 0
@@ -1336,18 +1399,7 @@ reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::t
                 umag = sqrt(ux * ux + uy * uy + uz * uz);
                 ph = nd.flow_p();
             }
-            s_phi.add(phi);
-            s_dcA.add(nd.dcA);
-            s_dcB.add(nd.dcB);
-            s_p.add(ph);
-            s_S.add(nd.S);
-            s_phit.add(nd.phit);
-            s_int.add(kint * phi * (R(1) - phi));                        // Eq. 67 integrand
-            ++nodes;
-            const bool finite = isfinite(phi) && isfinite(nd.dcA) && isfinite(nd.dcB) && isfinite(ph) &&
-                                isfinite(nd.S) && isfinite(umag) && isfinite(nd.phit);
-            bad += finite ? 0 : 1;
-            if (isfinite(umag)) umax = umag > umax ? umag : umax;
+            sums.add(phi, nd.dcA, nd.dcB, ph, nd.S, nd.phit, umag, kint);
             if constexpr (kTwoD<LAT>) quads += euler_quads4(phi_field, int(x), int(y), P);
             on = phi >= R(0.5);
         }
@@ -1358,41 +1410,159 @@ reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::t
             }
         }
     }
-    double acc[LBM_NRED_DEV];
-    acc[0] = s_phi.value();
-    acc[1] = s_dcA.value() + double(nodes) * P.c0[0];
-    acc[2] = s_dcB.value() + double(nodes) * P.c0[1];
-    acc[3] = s_p.value();
-    acc[4] = s_S.value();
-    acc[5] = double(umax);
-    acc[6] = s_phit.value();
-    acc[7] = double(bad);
-    acc[8] = s_int.value();
-    acc[9] = 0.25 * double(quads);
-    // block reduction: warp shuffles, then one warp over the warp results
-    __shared__ double sm[LBM_NRED_DEV][32];
-#pragma unroll
-    for (int i = 0; i < LBM_NRED_DEV; ++i) {
-        double v = acc[i];
-        for (int o = 16; o > 0; o >>= 1) {
-            const double u = __shfl_down_sync(0xffffffffu, v, o);
-            v = (i == 5) ? fmax(v, u) : v + u;
-        }
-        if (lane == 0) sm[i][warp] = v;
+    sums.write(0.25 * double(quads), threadIdx.x, blockIdx.x, P, partials);
+}
+
+// The diagnostics of a whole D3Q7 flow lattice in one read of the state (FP32 arithmetic): the
+// blocks march along z as in fused_flow_kernel, with phi of three planes and a one-node halo in
+// shared memory, so that neither a phi pass (88 B a node) nor a bit field of phi >= 1/2 and a
+// pass over it are needed. Blocks take items, a tile's chunk of planes, in turn; each writes one
+// row of partials. Bound by the latency of the gathers, like that kernel. lbm_reduce of a 384^3
+// FP32 state: 3.39 ms in three passes, 2.34 ms so (256^3 in place 0.97 -> 0.63 ms; FP16 384^3
+// 3.30 -> 3.20 ms). Four blocks an SM with FP32 storage (three: 2.52 ms), three with 16-bit
+// storage, where four spill (BF16 in place 208 x 176 x 297: 0.80 against 0.54 ms).
+template <class T, int MODE>
+__global__ void __launch_bounds__(FT, is16<T>() ? 3 : 4)
+reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ partials, int zchunk) {
+    using R = typename RealOf<T>::type;
+    __shared__ R ring[4][FY + 2][FX + 2];
+    __shared__ float fring[is16<T>() ? 4 : 1][FY + 2][FX + 2];         // f_0 / w_0 (16-bit storage)
+    __shared__ R park[2][4][FT];                                       // S, c - c_0^eq, phi~ of two planes
+    constexpr float kInvW0 = float(1.0 / D3Q19::w(0));
+    const float* f0 = is16<T>() ? st.rest + Addr<MODE>::kF0In * P.plane : nullptr;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * FX + tx;
+    const int tiles_x = (P.nx + FX - 1) / FX, tiles_y = (P.ny + FY - 1) / FY;
+    const int items = tiles_x * tiles_y * ((P.nz + zchunk - 1) / zchunk);
+    const R kint = R(4.0 / P.W);
+    const int sxy = P.nx * P.ny;
+    NodeSums<R> sums;
+    long long euler = 0;
+    int hxp = 0, hyp = 0;
+    if (tid < kHalo) {
+        if (tid < FX + 2) { hxp = tid - 1; hyp = -1; }
+        else if (tid < 2 * (FX + 2)) { hxp = tid - (FX + 2) - 1; hyp = FY; }
+        else if (tid < 2 * (FX + 2) + FY) { hxp = -1; hyp = tid - 2 * (FX + 2); }
+        else { hxp = FX; hyp = tid - 2 * (FX + 2) - FY; }
     }
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int bx = item % tiles_x, by = (item / tiles_x) % tiles_y, bz = item / (tiles_x * tiles_y);
+        const int x0 = bx * FX, y0 = by * FY, zs = bz * zchunk, ze = min(zs + zchunk, P.nz);
+        const int x = x0 + tx, y = y0 + ty;
+        const bool active = x < P.nx && y < P.ny;
+        // lattice column of a ring position: periodic wrap, mirror across x walls
+        auto column = [&](int hx, int hy, int& gx, int& gy) {
+            gx = x0 + hx;
+            gy = y0 + hy;
+            if (gx < 0) gx = P.wall_x ? 0 : gx + P.nx;
+            else if (gx >= P.nx) gx = P.wall_x ? P.nx - 1 : gx - P.nx;
+            if (gy < 0) gy += P.ny;
+            else if (gy >= P.ny) gy -= P.ny;
+            return gx >= 0 && gx < P.nx && gy >= 0 && gy < P.ny;
+        };
+        int ox, oy, hgx = 0, hgy = 0;
+        const bool own_ok = column(tx, ty, ox, oy);
+        const bool halo_ok = tid < kHalo && column(hxp, hyp, hgx, hgy);
+        Addr<MODE> own, halo;
+        own.nb.init_xy(ox, oy, P);
+        halo.nb.init_xy(hgx, hgy, P);
+        const bool xy_inner = x0 >= 2 && x0 + FX + 2 <= P.nx && y0 >= 2 && y0 + FY + 2 <= P.ny;
+        auto inner_plane = [&](int zr) { return xy_inner && zr >= 1 && zr <= P.nz - 2; };
+        auto zwrap = [&](int zz) {
+            if (zz < 0) return P.wall_z ? 0 : zz + P.nz;
+            if (zz >= P.nz) return P.wall_z ? P.nz - 1 : zz - P.nz;
+            return zz;
+        };
+        auto fill = [&](auto fast, int zz, bool keep) {
+            constexpr bool kFast = decltype(fast)::value;
+            const int zr = zwrap(zz), s = zz & 3;
+            auto phi_of = [&](Addr<MODE>& ad, int gx, int gy, bool ok, int rx, int ry, bool own_node) {
+                R v = R(0);
+                float r0 = 0.f;
+                if (ok) {
+                    const int node = node_of(gx, gy, zr, P);
+                    Node<T, LAT_D3Q7, false> nd;
+                    if constexpr (kFast) {
+                        nd.gather_scalars(st, AddrInner<MODE>{node, P.nx, sxy}, P);
+                    } else {
+                        ad.self = node;
+                        ad.nb.set_z(zr, P);
+                        nd.gather_scalars(st, ad, P);
+                    }
+                    nd.moments(P);
+                    v = nd.phi();
+                    if (own_node) {
+                        R (*pk)[FT] = park[zz & 1];
+                        pk[0][tid] = nd.S;
+                        pk[1][tid] = nd.dcA;
+                        pk[2][tid] = nd.dcB;
+                        pk[3][tid] = nd.phit;
+                    }
+                    if constexpr (is16<T>()) r0 = f0[node] * kInvW0;
+                }
+                ring[s][ry][rx] = v;
+                if constexpr (is16<T>()) fring[s][ry][rx] = r0;
+            };
+            phi_of(own, ox, oy, own_ok, tx + 1, ty + 1, keep && active);
+            if (tid < kHalo) phi_of(halo, hgx, hgy, halo_ok, hxp + 1, hyp + 1, false);
+        };
+        auto fill_any = [&](int zz, bool keep) {
+            if (inner_plane(zwrap(zz))) fill(std::true_type{}, zz, keep);
+            else fill(std::false_type{}, zz, keep);
+        };
+        auto centre = [&](const auto& ad, int z) {
+            const int sp = (z - 1) & 3, sc = z & 3, sn = (z + 1) & 3;
+            Node<T, LAT_D3Q7, true> nd;
+            nd.gather_flow(st, ad, P, [&](int k, int ex, int ey, int ez, Slot) {
+                if (k == 0 || ad.writer(k, ex, ey, ez) == ad.self) return fring[is16<T>() ? sc : 0][ty + 1][tx + 1];
+                return fring[is16<T>() ? (ez > 0 ? sp : (ez < 0 ? sn : sc)) : 0][ty + 1 - ey][tx + 1 - ex];
+            });
+            const R phi = ring[sc][ty + 1][tx + 1];
+            R gx, gy, gz, lap, Fx, Fy, Fz, ux, uy, uz;
+            stencil([&](int dx, int dy, int dz) {
+                        return ring[dz < 0 ? sp : (dz > 0 ? sn : sc)][ty + 1 + dy][tx + 1 + dx];
+                    }, phi, gx, gy, gz, lap);
+            force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
+            const R (*pk)[FT] = park[z & 1];
+            sums.add(phi, pk[1][tid], pk[2][tid], nd.flow_p(), pk[0][tid], pk[3][tid],
+                     sqrt(ux * ux + uy * uy + uz * uz), kint);
+            // cell positions this node owns (see euler_cells): its own, and at the far wall of a
+            // walled axis the one past it
+            const int x1 = (P.wall_x && x == P.nx - 1) ? 1 : 0, z1 = (P.wall_z && z == P.nz - 1) ? 1 : 0;
+            for (int dz = 0; dz <= z1; ++dz)
+                for (int dx = 0; dx <= x1; ++dx) {
+                    int b[2][2][2];
 #pragma unroll
-        for (int i = 0; i < LBM_NRED_DEV; ++i) {
-            double v = lane < nw ? sm[i][lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) {
-                const double u = __shfl_down_sync(0xffffffffu, v, o);
-                v = (i == 5) ? fmax(v, u) : v + u;
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+                            for (int a = 0; a < 2; ++a) {
+                                const int ax = dx + a - 1, az = dz + c - 1;
+                                const bool out = (P.wall_x && (x + ax < 0 || x + ax >= P.nx)) ||
+                                                 (P.wall_z && (z + az < 0 || z + az >= P.nz));
+                                b[c][bb][a] = !out && ring[(z + az) & 3][ty + bb][tx + 1 + ax] >= R(0.5);
+                            }
+                    euler += euler_of_cells(b);
+                }
+        };
+        __syncthreads();                       // the ring of the item before is read no more
+        fill_any(zs - 1, false);
+        fill_any(zs, true);
+        for (int z = zs; z < ze; ++z) {
+            fill_any(z + 1, z + 1 < ze);
+            __syncthreads();
+            if (active) {
+                if (inner_plane(z)) {
+                    centre(AddrInner<MODE>{node_of(x, y, z, P), P.nx, sxy}, z);
+                } else {
+                    own.self = node_of(x, y, z, P);
+                    own.nb.set_z(z, P);
+                    centre(own, z);
+                }
             }
-            if (lane == 0) partials[(long long)blockIdx.x * LBM_NRED_DEV + i] = v;
         }
     }
+    sums.write(double(euler), tid, blockIdx.x, P, partials);
 }
 
 // Planes (rows, in 2D) a marching block goes through: the count, at most 32, for which the
@@ -1560,6 +1730,23 @@ struct Launchers {
                        double* partials, int nblocks, cudaStream_t s) {
         R* phi = static_cast<R*>(phi_work);
         unsigned* bits = static_cast<unsigned*>(bits_work);
+        // a whole flow lattice with D3Q7 sets and FP32 arithmetic (a slab, which has no bit field,
+        // keeps the neighbours' phi in the phi field; FP64 halos would cost the FP64 pipe)
+        if constexpr (FLOW && LAT == LAT_D3Q7 && sizeof(R) == 4) {
+            if (bits) {
+                int nb = nblocks;
+                const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
+                LBM_MODE_SWITCH(mode, {
+                    nb = resident_blocks(reduce_march_kernel<T, M>, nblocks);
+                    const int zc = march_chunk(tiles, P.nz, nb, 0.7);
+                    reduce_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, partials, zc);
+                });
+                if (nb < nblocks)
+                    cudaMemsetAsync(partials + (size_t)nb * LBM_NRED_DEV, 0,
+                                    (size_t)(nblocks - nb) * LBM_NRED_DEV * sizeof(double), s);
+                return;
+            }
+        }
         if constexpr (FLOW || kTwoD<LAT>) {
             Launchers::template phi<LAT>(P, st, mode, phi_work, s);
         }
