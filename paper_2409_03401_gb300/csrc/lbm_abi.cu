@@ -370,7 +370,7 @@ void launch_one(lbm_ctx* c, int64_t t, cudaEvent_t* e) {
     }
     if (e) cudaEventRecord(e[1], c->stream);
     if (fused) {
-        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, c->stream);
+        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, c->slab ? nullptr : c->work + c->L.off_phi, c->stream);
     } else {
         LBM_DISPATCH(c->p.storage, launch_step, c->dp, src, dst, c->p.lattice, c->p.flow != 0, mode,
                      c->work + c->L.off_phi, c->stream);
@@ -499,7 +499,9 @@ lbm_status lbm_profile_end(lbm_ctx* c, double* out) {
 }
 
 int lbm_kernels_per_step(const lbm_ctx* c) {
-    return c ? ((c->p.flow && !one_pass(c)) ? 2 : 1) : 0;
+    if (!c) return 0;
+    const bool rim_pass = one_pass(c) && c->p.storage == LBM_F32 && !c->slab && lbm::flow_tma_applies(c->dp);
+    return (c->p.flow && !one_pass(c)) || rim_pass ? 2 : 1;
 }
 
 int64_t lbm_time(const lbm_ctx* c) { return c ? c->t : -1; }
@@ -556,7 +558,7 @@ lbm_status lbm_step_buffers(const lbm_params* p, const void* d_src, void* d_dst,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaGetLastError();
     if (L.two && fused_flow(p)) {
-        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, s);
+        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, nullptr, s);
     } else {
         const int mode = L.two ? lbm::kModePull : ((t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven);
         char* phi = static_cast<char*>(d_work) + L.off_phi;

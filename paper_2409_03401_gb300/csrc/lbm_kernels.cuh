@@ -1565,13 +1565,13 @@ reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ 
     sums.write(double(euler), tid, blockIdx.x, P, partials);
 }
 
-// Planes (rows, in 2D) a marching block goes through: the count, at most 32, for which the
+// Planes (rows, in 2D) a marching block goes through: the count, up to ``most``, for which the
 // waves of blocks over the chip's ``slots`` times the planes each block computes, ``extra`` for
 // the planes around the chunk among them, are fewest.
-inline int march_chunk(long long tiles, int n, long long slots, double extra) {
+inline int march_chunk(long long tiles, int n, long long slots, double extra, int most = 32) {
     int best = 1;
     double cost = 1e300;
-    for (int c = 1; c <= n && c <= 32; ++c) {
+    for (int c = 1; c <= n && c <= most; ++c) {
         const long long blocks = tiles * ((n + c - 1) / c);
         const double t = double((blocks + slots - 1) / slots) * (c + extra);
         if (t <= cost) { cost = t; best = c; }
@@ -1582,6 +1582,7 @@ inline int march_chunk(long long tiles, int n, long long slots, double extra) {
 }  // namespace lbm
 
 #include "lbm_two_steps.cuh"
+#include "lbm_flow_tma.cuh"
 
 namespace lbm {
 
@@ -1663,7 +1664,33 @@ struct Launchers {
     static void two_steps(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
         launch_two_steps_at<T, LAT>(P, src, dst, s);
     }
-    static void fused(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
+    template <int COLL>
+    static bool flow_tma(const DevParams& P, const StateView& src, const StateView& dst, R* phi, cudaStream_t s) {
+        if constexpr (std::is_same<T, float>::value) {
+            tma::Maps maps;
+            if (!tma_maps(P, src, maps)) return false;
+            if (cudaFuncSetAttribute(flow_tma_kernel<COLL>, cudaFuncAttributeMaxDynamicSharedMemorySize, tma::kSmem) !=
+                cudaSuccess) {
+                cudaGetLastError();
+                return false;
+            }
+            const dim3 tiles((P.nx + tma::X - 1) / tma::X, (P.ny + tma::Y - 1) / tma::Y);
+            // 20 to 24 planes measured best (512^3: 7.39 ms a step; 12: 7.51, 32: 8.19)
+            const int zc = march_chunk((long long)tiles.x * tiles.y, P.nz, 152, 3.0, 24);
+            launch_after_previous<R>(rim_phi_kernel, dim3((2 * (P.nx + P.ny - 2) + kBlockX - 1) / kBlockX, 1, P.nz),
+                                     dim3(kBlockX), 0, s, P, src, phi);
+            launch_after_previous<R>(flow_tma_kernel<COLL>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(tma::T),
+                                     size_t(tma::kSmem), s, P, maps, src, dst, phi, zc);
+            return true;
+        }
+        return false;
+    }
+    // ``phi_work``: a phi field to use as scratch, or nullptr
+    static void fused(const DevParams& P, const StateView& src, const StateView& dst, void* phi_work, cudaStream_t s) {
+        if (std::is_same<T, float>::value && phi_work && flow_tma_applies(P)) {
+            R* phi = static_cast<R*>(phi_work);
+            if (P.coll == 2 ? flow_tma<2>(P, src, dst, phi, s) : flow_tma<0>(P, src, dst, phi, s)) return;
+        }
         const dim3 block(FX, FY);
         const int zchunk = march_chunk((long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY), P.z_hi - P.z_lo,
                                        152 * fused_min_blocks<T, 0>(), 0.7);
@@ -1808,8 +1835,8 @@ struct Launchers {
         }                                                                                                 \
     }                                                                                                     \
     void launch_fused_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst,            \
-                               cudaStream_t s) {                                                          \
-        Launchers<T>::fused(P, src, dst, s);                                                              \
+                               void* phi_work, cudaStream_t s) {                                          \
+        Launchers<T>::fused(P, src, dst, phi_work, s);                                                    \
     }                                                                                                     \
     void launch_fields_##SUFFIX(const DevParams& P, const StateView& st, int lat, bool flow, int mode,    \
                                 void* phi, FieldPtrs out, cudaStream_t s) {                               \

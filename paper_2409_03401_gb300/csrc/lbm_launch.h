@@ -16,6 +16,16 @@ struct FieldPtrs { void* p[LBM_NFIELDS_DEV]; };
 // streaming modes (see lbm_kernels.cuh)
 constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
 
+// Whether an FP32 two-buffer flow step on D3Q7 sets takes the TMA-staged kernel (given a phi field
+// as scratch): rows of whole 16-byte pieces (a tensor copy's rule), the undivided lattice, no
+// walls in x, and 30 million nodes, so that the tiles at the lattice's ends are few enough for
+// what they cost more (512^3: 7.39 against 8.19 ms a step, 384^3: 3.20 against 3.46 ms, 256^3:
+// 1.05 against 1.04 ms, 192^3: 0.49 against 0.44 ms).
+inline bool flow_tma_applies(const DevParams& P) {
+    return P.nx % 4 == 0 && P.nx >= 64 && P.ny >= 32 && P.n >= 30000000 && !P.wall_x && P.z_lo == 0 && P.z_hi == P.nz &&
+           P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z;
+}
+
 #define LBM_DECLARE_LAUNCHERS(SUFFIX)                                                                   \
     void launch_init_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, bool pull,         \
                               const double*, const double*, const double*, cudaStream_t);                \
@@ -27,7 +37,8 @@ constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
                               int mode, void* phi, cudaStream_t);                                        \
     void launch_two_steps_##SUFFIX(const DevParams&, const StateView&, const StateView&, int lat,        \
                                    cudaStream_t);                                                         \
-    void launch_fused_##SUFFIX(const DevParams&, const StateView&, const StateView&, cudaStream_t);       \
+    void launch_fused_##SUFFIX(const DevParams&, const StateView&, const StateView&, void* phi_work,      \
+                               cudaStream_t);                                                            \
     void launch_fields_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, int mode,        \
                                 void* phi, FieldPtrs, cudaStream_t);                                     \
     void launch_reduce_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, int mode,        \

@@ -34,6 +34,14 @@ def test_two_buffer_flow_step_matches_the_fused_kernel(storage, shape, collision
     _compare_with_fused(LBMParams(*shape, flow=True, storage=storage, collision=collision, wall_z=wall_z), 5)
 
 
+@pytest.mark.parametrize("shape", [(64, 700, 671), (100, 601, 500), (1024, 32, 917), (512, 243, 242)])
+@pytest.mark.parametrize("collision,wall_z", [("BGK", True), ("BGK", False), ("TRT", False), ("MRT", True)])
+def test_tma_staged_flow_step_matches_the_fused_kernel(shape, collision, wall_z):
+    # from 30 million nodes on, rows of whole 16-byte pieces: the step's loads come by tensor copies,
+    # the lattice's ends apart; tiles of 32 x 15 nodes, the last ones overlapping, several chunks
+    _compare_with_fused(LBMParams(*shape, flow=True, collision=collision, wall_z=wall_z), 3)
+
+
 def test_fp32_flow_step_on_both_sides_of_the_size_rule():
     _compare_with_fused(LBMParams(100, 75, 79, flow=True, wall_z=True), 4)       # 592,500 nodes: two passes
     _compare_with_fused(LBMParams(100, 75, 81, flow=True, wall_z=True), 4)       # 607,500: the fused kernel
