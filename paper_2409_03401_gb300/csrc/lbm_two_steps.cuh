@@ -6,7 +6,7 @@
 // is collide_at_rest in both steps, so the result equals two calls of step_kernel bit for bit.
 //
 // A single step is bound by HBM (168 B a node on D3Q7, at 0.97 of the copy bandwidth); two steps
-// a pass halve that traffic. Measured a step: 4096^2 D2Q9 543 -> 323 us, 256^3 D3Q7 423 -> 316 us.
+// a pass halve that traffic. Measured a step: 4096^2 D2Q9 543 -> 323 us, 256^3 D3Q7 423 -> 297 us.
 // What the results move along x goes through shuffles before it is stored, so that every warp
 // writes whole rows at its own x: stores shifted by a node leave partial sectors in a buffer
 // that is not the one just read, and a copy in that pattern runs at 4.9 instead of 6.3 TB/s.
@@ -84,6 +84,24 @@ __device__ __forceinline__ void collide_second(const typename RealOf<T>::type (&
 
 __device__ __forceinline__ int wrapped(int q, int n) { return ((q % n) + n) % n; }
 
+// A barrier of the block in shared memory, and a wait of a bounded number of tries for its phase.
+__device__ __forceinline__ void block_barrier_init(unsigned b, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(count) : "memory");
+}
+__device__ __forceinline__ void block_barrier_arrive(unsigned b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+}
+__device__ __forceinline__ bool block_barrier_wait(unsigned b, unsigned parity) {
+    for (int i = 0; i < (1 << 20); ++i) {
+        unsigned done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(b), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
 // 3D: a block of 32 x 16 threads marches along z; its 28 x 14 inner threads own nodes, the
 // outer ring computes the first collision of the tile's neighbours again.
 constexpr int T2X = 32, T2Y = 16, T2IX = T2X - 4, T2IY = T2Y - 2;
@@ -95,9 +113,12 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
     begin_after_previous();
     using R = typename RealOf<T>::type;
     constexpr int Q = 7;
-    // populations moving along y, of three planes: the plane being assembled, the next one,
-    // and the one that threads ahead of the slowest (by one barrier) already write
-    __shared__ R ys[3][6][T2Y][T2X];
+    // populations moving along y, of four planes, and a barrier for each that all warps reach when
+    // theirs are written (256^3: 297 us a step; 321 with one __syncthreads a plane). A plane's are read a plane later, so that a warp seldom waits; a warp
+    // that has seen a barrier knows that all have read what it overwrites two planes on.
+    extern __shared__ __align__(16) unsigned char t2_smem[];
+    R (*ys)[6][T2Y][T2X] = reinterpret_cast<R (*)[6][T2Y][T2X]>(t2_smem);
+    const unsigned bars = unsigned(__cvta_generic_to_shared(t2_smem)) + 4 * 6 * T2Y * T2X * sizeof(R);
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int x = int(blockIdx.x) * T2IX + tx - 2, y = int(blockIdx.y) * T2IY + ty - 1;
     const int zs = blockIdx.z * zchunk, ze = min(zs + zchunk, P.nz);
@@ -110,6 +131,11 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
     const bool wall_lo = P.wall_x && x == 0, wall_hi = P.wall_x && x == P.nx - 1;
     // columns of the neighbours along y
     const int cyp = (gy + 1 == P.ny ? 0 : gy + 1) * P.nx + gx, cym = (gy == 0 ? P.ny - 1 : gy - 1) * P.nx + gx;
+
+    if (tx == 0 && ty == 0)
+        for (int i = 0; i < 4; ++i) block_barrier_init(bars + 8 * i, T2Y);
+    __syncthreads();
+    bool ok = true;  // no wait ran out
 
     R in[3][Q];      // incoming populations of plane z (second step); +z from z - 1 in slot 5
     R up[3];         // moving +z out of plane z
@@ -127,10 +153,12 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
             o[s][1] = wall_lo ? o[s][2] : a;
             o[s][2] = wall_hi ? own : b;
         }
+        __syncwarp();
+        if (tx == 0 && zz >= zs) block_barrier_arrive(bars + 8 * slot);   // nobody reads plane zs - 1
     };
     int slot = 0;
     if (zs > 0 || !P.wall_z) {
-        first(zs - 1, 2);
+        first(zs - 1, 3);
 #pragma unroll
         for (int s = 0; s < 3; ++s) in[s][5] = o[s][5];
         first(zs, slot);
@@ -145,10 +173,10 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
         up[s] = o[s][5];
     }
     for (int z = zs; z < ze; ++z) {
-        const int next = slot == 2 ? 0 : slot + 1;
+        const int next = (slot + 1) & 3;
         const bool top = P.wall_z && z == P.nz - 1, low = P.wall_z && z == 0;
         if (!top) first(z + 1, next);
-        __syncthreads();
+        if (ok) ok = block_barrier_wait(bars + 8 * slot, unsigned(z - zs) / 4 & 1);
         if (row_in) {
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
@@ -156,6 +184,7 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
                 in[s][4] = ys[slot][2 * s + 1][ty + 1][tx];
                 in[s][6] = top ? up[s] : o[s][6];
             }
+            if (!ok) in[1][0] = __int_as_float(0x7fc00000);            // never in a run: the state shows it
             const int zp = z + 1 == P.nz ? 0 : z + 1, zm = z == 0 ? P.nz - 1 : z - 1;
             const int self = z * nxy + col;
             collide_second<T, LAT_D3Q7>(in, dst, self, inner, wall_lo, wall_hi, P, [&](int k) -> Slot {
@@ -259,8 +288,10 @@ void launch_two_steps_at(const DevParams& P, const StateView& src, const StateVi
     if constexpr (LAT == LAT_D3Q7) {
         const dim3 tiles((P.nx + T2IX - 1) / T2IX, (P.ny + T2IY - 1) / T2IY);
         const int zc = march_chunk((long long)tiles.x * tiles.y, P.nz, 152 * kTwoStepsBlocks, 2.0);
-        launch_after_previous<float>(two_steps_3d_kernel<T>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(T2X, T2Y), 0, s, P,
-                              src, dst, zc);
+        constexpr int smem = 4 * 6 * T2Y * T2X * int(sizeof(float)) + 64;
+        cudaFuncSetAttribute(two_steps_3d_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        launch_after_previous<float>(two_steps_3d_kernel<T>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(T2X, T2Y),
+                                     size_t(smem), s, P, src, dst, zc);
     } else {
         const int wins = (P.nx + T2IX - 1) / T2IX, bx = (wins + T2Warps - 1) / T2Warps;
         const int yc = march_chunk(bx, P.ny, 152 * kTwoSteps2DBlocks, 2.0);
