@@ -1435,17 +1435,18 @@ reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::t
     sums.write(0.25 * double(quads), threadIdx.x, blockIdx.x, P, partials);
 }
 
-// The diagnostics of a whole D3Q7 flow lattice in one read of the state (FP32 arithmetic): the
-// blocks march along z as in fused_flow_kernel, with phi of three planes and a one-node halo in
-// shared memory, so that neither a phi pass (88 B a node) nor a bit field of phi >= 1/2 and a
-// pass over it are needed. Blocks take items, a tile's chunk of planes, in turn; each writes one
-// row of partials. Bound by the latency of the gathers, like that kernel. lbm_reduce of a 384^3
-// FP32 state: 3.39 ms in three passes, 2.34 ms so (256^3 in place 0.97 -> 0.63 ms; FP16 384^3
-// 3.30 -> 3.20 ms). Four blocks an SM with FP32 storage (three: 2.52 ms), three with 16-bit
-// storage, where four spill (BF16 in place 208 x 176 x 297: 0.80 against 0.54 ms).
-template <class T, int MODE>
-__global__ void __launch_bounds__(FT, is16<T>() ? 3 : 4)
-reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ partials, int zchunk) {
+// Lattices from which on diagnostics and fields march; in smaller ones the planes, one after
+// another, take longer than the launches of the passes (46 x 144 x 33: 93 against 78 us).
+constexpr long long kMarchNodes = 600000;
+
+// One read of the state of a whole D3Q7 flow lattice (FP32 arithmetic): the blocks march along z
+// as in fused_flow_kernel, with phi of three planes and a one-node halo in shared memory, so that
+// no phi pass (88 B a node) is needed. Blocks take items, a tile's chunk of planes, in turn. For
+// every node ``sink(node, x, y, z, nd, phi, kept, u, on)`` gets its flow populations, phi, S, c -
+// c_0^eq (two) and phi~ (kept[0..3]), u, and a functor that reads phi of a neighbour. Bound by the
+// latency of the gathers, like that kernel.
+template <class T, int MODE, class Sink>
+__device__ __forceinline__ void march_nodes(const DevParams& P, const StateView& st, int zchunk, Sink sink) {
     using R = typename RealOf<T>::type;
     __shared__ R ring[4][FY + 2][FX + 2];
     __shared__ float fring[is16<T>() ? 4 : 1][FY + 2][FX + 2];         // f_0 / w_0 (16-bit storage)
@@ -1455,10 +1456,7 @@ reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * FX + tx;
     const int tiles_x = (P.nx + FX - 1) / FX, tiles_y = (P.ny + FY - 1) / FY;
     const int items = tiles_x * tiles_y * ((P.nz + zchunk - 1) / zchunk);
-    const R kint = R(4.0 / P.W);
     const int sxy = P.nx * P.ny;
-    NodeSums<R> sums;
-    long long euler = 0;
     int hxp = 0, hyp = 0;
     if (tid < kHalo) {
         if (tid < FX + 2) { hxp = tid - 1; hyp = -1; }
@@ -1544,28 +1542,13 @@ reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ 
                         return ring[dz < 0 ? sp : (dz > 0 ? sn : sc)][ty + 1 + dy][tx + 1 + dx];
                     }, phi, gx, gy, gz, lap);
             force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
-            const R (*pk)[FT] = park[z & 1];
-            sums.add(phi, pk[1][tid], pk[2][tid], nd.flow_p(), pk[0][tid], pk[3][tid],
-                     sqrt(ux * ux + uy * uy + uz * uz), kint);
-            // cell positions this node owns (see euler_cells): its own, and at the far wall of a
-            // walled axis the one past it
-            const int x1 = (P.wall_x && x == P.nx - 1) ? 1 : 0, z1 = (P.wall_z && z == P.nz - 1) ? 1 : 0;
-            for (int dz = 0; dz <= z1; ++dz)
-                for (int dx = 0; dx <= x1; ++dx) {
-                    int b[2][2][2];
+            R kept[4];
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
-#pragma unroll
-                        for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-                            for (int a = 0; a < 2; ++a) {
-                                const int ax = dx + a - 1, az = dz + c - 1;
-                                const bool out = (P.wall_x && (x + ax < 0 || x + ax >= P.nx)) ||
-                                                 (P.wall_z && (z + az < 0 || z + az >= P.nz));
-                                b[c][bb][a] = !out && ring[(z + az) & 3][ty + bb][tx + 1 + ax] >= R(0.5);
-                            }
-                    euler += euler_of_cells(b);
-                }
+            for (int i = 0; i < 4; ++i) kept[i] = park[z & 1][i][tid];
+            const R u[3] = {ux, uy, uz};
+            sink(ad.self, x, y, z, nd, phi, kept, u, [&](int dx, int dy, int dz) {
+                return ring[(z + dz) & 3][ty + 1 + dy][tx + 1 + dx];
+            });
         };
         __syncthreads();                       // the ring of the item before is read no more
         fill_any(zs - 1, false);
@@ -1584,7 +1567,67 @@ reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ 
             }
         }
     }
-    sums.write(double(euler), tid, blockIdx.x, P, partials);
+}
+
+// The diagnostics of such a lattice, one row of partials a block, without the bit field of phi >=
+// 1/2 and the pass over it. lbm_reduce of a 384^3 FP32 state: 3.39 ms in three passes, 2.34 ms so
+// (256^3 in place 0.97 -> 0.63 ms; FP16 384^3 3.30 -> 3.20 ms). Four blocks an SM with FP32 storage
+// (three: 2.52 ms), three with 16-bit storage, where four spill (BF16 in place 208 x 176 x 297:
+// 0.80 against 0.54 ms).
+template <class T, int MODE>
+__global__ void __launch_bounds__(FT, is16<T>() ? 3 : 4)
+reduce_march_kernel(const DevParams P, const StateView st, double* __restrict__ partials, int zchunk) {
+    using R = typename RealOf<T>::type;
+    const R kint = R(4.0 / P.W);
+    NodeSums<R> sums;
+    long long euler = 0;
+    march_nodes<T, MODE>(P, st, zchunk, [&](int, int x, int, int z, const auto& nd, R phi, const R* kept, const R* u,
+                                            auto at) {
+        sums.add(phi, kept[1], kept[2], nd.flow_p(), kept[0], kept[3], sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]),
+                 kint);
+        // cell positions this node owns (see euler_cells): its own, and at the far wall of a
+        // walled axis the one past it
+        const int x1 = (P.wall_x && x == P.nx - 1) ? 1 : 0, z1 = (P.wall_z && z == P.nz - 1) ? 1 : 0;
+        for (int dz = 0; dz <= z1; ++dz)
+            for (int dx = 0; dx <= x1; ++dx) {
+                int b[2][2][2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) {
+                            const int ax = dx + a - 1, az = dz + c - 1;
+                            const bool out = (P.wall_x && (x + ax < 0 || x + ax >= P.nx)) ||
+                                             (P.wall_z && (z + az < 0 || z + az >= P.nz));
+                            b[c][bb][a] = !out && at(ax, bb - 1, az) >= R(0.5);
+                        }
+                euler += euler_of_cells(b);
+            }
+    });
+    sums.write(double(euler), threadIdx.y * FX + threadIdx.x, blockIdx.x, P, partials);
+}
+
+// The fields of such a lattice (see fields_kernel): seven fields of a 512^3 FP32 state 6.94 -> 6.24
+// ms, 256^3 in place 0.74 -> 0.61 ms.
+template <class T, int MODE>
+__global__ void __launch_bounds__(FT, is16<T>() ? 3 : 4)
+fields_march_kernel(const DevParams P, const StateView st, FieldPtrs out, int zchunk) {
+    using R = typename RealOf<T>::type;
+    march_nodes<T, MODE>(P, st, zchunk, [&](int node, int, int, int, const auto& nd, R phi, const R* kept, const R* u, auto) {
+        const R p = interp_p(phi);
+        auto put = [&](int i, R v) { if (out.p[i]) static_cast<R*>(out.p[i])[node] = v; };
+        put(0, phi);
+        put(1, closure_dev(kept[1], p, 0, P));
+        put(2, closure_dev(kept[2], p, 1, P));
+        put(3, kept[1] + coef<R>(P).c0[0]);
+        put(4, kept[2] + coef<R>(P).c0[1]);
+        put(5, nd.flow_p());
+        put(6, u[0]);
+        put(7, u[1]);
+        put(8, u[2]);
+        put(9, kept[0]);
+    });
 }
 
 // Planes (rows, in 2D) a marching block goes through: the count, up to ``most``, for which the
@@ -1753,6 +1796,19 @@ struct Launchers {
     template <int LAT, bool FLOW>
     static void fields(const DevParams& P, const StateView& st, int mode, void* phi_work, FieldPtrs out,
                        cudaStream_t s) {
+        // as in reduce(); a slab's planes end beside ghost planes, and 16-bit storage is faster in
+        // two passes (384^3 FP16: 2.24 against 2.92 ms)
+        if constexpr (FLOW && LAT == LAT_D3Q7 && std::is_same<T, float>::value) {
+            if (P.n >= kMarchNodes && P.z_lo == 0 && P.z_hi == P.nz && P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z) {
+                const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
+                LBM_MODE_SWITCH(mode, {
+                    const int nb = resident_blocks(fields_march_kernel<T, M>, 152 * 8);
+                    const int zc = march_chunk(tiles, P.nz, nb, 0.7);
+                    fields_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, out, zc);
+                });
+                return;
+            }
+        }
         int bx; const dim3 grid = node_grid(P, bx);
         R* phi = static_cast<R*>(phi_work);
         if constexpr (FLOW) Launchers::template phi<LAT>(P, st, mode, phi_work, s);
@@ -1782,7 +1838,7 @@ struct Launchers {
         // a whole flow lattice with D3Q7 sets and FP32 arithmetic (a slab, which has no bit field,
         // keeps the neighbours' phi in the phi field; FP64 halos would cost the FP64 pipe)
         if constexpr (FLOW && LAT == LAT_D3Q7 && sizeof(R) == 4) {
-            if (bits) {
+            if (bits && P.n >= kMarchNodes) {
                 int nb = nblocks;
                 const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
                 LBM_MODE_SWITCH(mode, {

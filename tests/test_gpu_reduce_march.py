@@ -16,7 +16,9 @@ from workloads.params import LBMParams
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(32, 8, 4), (33, 9, 37), (31, 7, 5), (64, 24, 33), (40, 1, 6), (1, 9, 3), (70, 30, 1)]
+# from 600,000 nodes on the lattice is read by the marching kernels, below in separate passes
+SHAPES = [(33, 9, 37), (40, 1, 6), (70, 30, 1), (96, 80, 80), (33, 135, 137), (1, 801, 750), (800, 1, 751),
+          (801, 750, 1)]
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
@@ -40,6 +42,6 @@ def test_sums_match_the_fields(storage, inplace, shape, wall_x, wall_z):
         umax = float(torch.sqrt(f["ux"] ** 2 + f["uy"] ** 2 + f["uz"] ** 2).max())
         assert abs(s["umax"] - umax) <= 1e-5 * umax
         assert s["nonfinite"] == 0
-        if p.nz > 1:                    # the oracle counts nz = 1 as a 2D lattice
+        if p.nz > 1 and p.nodes < 700000:      # the oracle counts nz = 1 as a 2D lattice
             assert s["euler"] == euler_characteristic(f["phi"].cpu().numpy(), walls=(wall_x, False, wall_z))
         sim.step(1)
