@@ -806,11 +806,17 @@ step_kernel(const DevParams P, const StateView st, const StateView out,
     step_node<T, LAT, FLOW, COLL>(ad, P, st, out, phi_field);
 }
 
+// A block set up by launch_after_previous costs the scheduler about 1 ns, a plain one 0.6: a phi
+// pass of many narrow 16-bit blocks is bound by that (48 x 354 x 160, 56,640 blocks of 64: 60 us
+// against 36), so blocks below kBlockX threads are launched the plain way above this number.
+constexpr long long kAfterBlocks = 8192;
+
 // phi = sum g + S/2 of every node (Eq. 49), read by the capillary stencil.
-template <class T, int LAT, int MODE>
+// AFTER: launched after a step kernel with launch_after_previous.
+template <class T, int LAT, int MODE, bool AFTER>
 __global__ void __launch_bounds__(kBlockX)
 phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* __restrict__ phi_out) {
-    begin_after_previous();
+    if constexpr (AFTER) begin_after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
     if (x >= P.nx) return;
@@ -1691,16 +1697,18 @@ struct Launchers {
         else init_kernel<T, LAT, FLOW, AA_EVEN><<<grid, bx, 0, s>>>(P, st, phi0, cA0, cB0);
     }
     // ``in_step``: the first kernel of a step (see begin_after_previous); the diagnostics' phi pass
-    // stands between kernels launched the plain way and is cheaper to queue like them
+    // stands between kernels launched the plain way and is cheaper to queue like them. FP16 steps
+    // of 48 x 354 x 160 with the pass after the previous kernel / plain: 209 / 191 us, in place
+    // 223 / 209; 128^3 in place (blocks of kBlockX): 130 / 132; 64^3 two copies: 17.9 / 19.7.
     template <int LAT>
     static void phi(const DevParams& P, const StateView& st, int mode, void* phi_work, cudaStream_t s,
                     bool in_step = false) {
         int bx; const dim3 grid = step_grid(P, bx);
         R* ph = static_cast<R*>(phi_work);
-        if (in_step) {
-            LBM_MODE_SWITCH(mode, launch_after_previous<R>(phi_kernel<T, LAT, M>, grid, dim3(bx), 0, s, P, st, ph));
+        if (in_step && (bx == kBlockX || (long long)grid.x * grid.y * grid.z <= kAfterBlocks)) {
+            LBM_MODE_SWITCH(mode, launch_after_previous<R>(phi_kernel<T, LAT, M, true>, grid, dim3(bx), 0, s, P, st, ph));
         } else {
-            LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M><<<grid, bx, 0, s>>>(P, st, ph));
+            LBM_MODE_SWITCH(mode, phi_kernel<T, LAT, M, false><<<grid, bx, 0, s>>>(P, st, ph));
         }
     }
     template <int LAT>

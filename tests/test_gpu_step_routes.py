@@ -34,6 +34,12 @@ def test_two_buffer_flow_step_matches_the_fused_kernel(storage, shape, collision
     _compare_with_fused(LBMParams(*shape, flow=True, storage=storage, collision=collision, wall_z=wall_z), 5)
 
 
+@pytest.mark.parametrize("storage", ["f16", "f32", "f64"])
+@pytest.mark.parametrize("shape", [(20, 128, 64), (20, 130, 70)])      # 8192 and 9100 narrow blocks
+def test_phi_pass_of_many_narrow_blocks(storage, shape):
+    _compare_with_fused(LBMParams(*shape, flow=True, storage=storage), 5)
+
+
 @pytest.mark.parametrize("shape", [(64, 700, 671), (100, 601, 500), (1024, 32, 917), (512, 243, 242)])
 @pytest.mark.parametrize("collision,wall_z", [("BGK", True), ("BGK", False), ("TRT", False), ("MRT", True)])
 def test_tma_staged_flow_step_matches_the_fused_kernel(shape, collision, wall_z):
