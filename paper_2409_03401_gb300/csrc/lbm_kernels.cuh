@@ -1441,8 +1441,9 @@ reduce_kernel(const DevParams P, const StateView st, const typename RealOf<T>::t
     sums.write(0.25 * double(quads), threadIdx.x, blockIdx.x, P, partials);
 }
 
-// Lattices from which on diagnostics and fields march; in smaller ones the planes, one after
-// another, take longer than the launches of the passes (46 x 144 x 33: 93 against 78 us).
+// Lattices from which on diagnostics and fields may march (march_planes); in smaller ones the
+// planes, one after another, take longer than the launches of the passes (46 x 144 x 33: 93
+// against 78 us).
 constexpr long long kMarchNodes = 600000;
 
 // One read of the state of a whole D3Q7 flow lattice (FP32 arithmetic): the blocks march along z
@@ -1649,6 +1650,21 @@ inline int march_chunk(long long tiles, int n, long long slots, double extra, in
     }
     return best;
 }
+// Planes per item of the marching diagnostics and fields on ``slots`` resident blocks, or 0 where
+// separate passes are faster: below kMarchNodes, and where the threads' turns, empty ones of
+// ragged tiles and of the last round among them, are many for each node. Turns a node and the
+// passes' time over the march's: FP32 sums 288x288x200 1.13, 1.38; 166x160x128 1.25, 1.22;
+// 48x200x200 1.48, 1.06; 40x240x240 1.70, 0.99; 33x300x300 2.12, 0.82; FP16 sums 288x288x200 1.06,
+// 1.27; 160x160x60 1.25, 1.12; 48x200x200 1.47, 0.95; 40x240x240 1.74, 0.83.
+template <class T>
+inline int march_planes(const DevParams& P, int slots) {
+    if (P.n < kMarchNodes) return 0;
+    const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
+    const int zc = march_chunk(tiles, P.nz, slots, is16<T>() ? 2.0 : 0.7);
+    const long long rounds = (tiles * ((P.nz + zc - 1) / zc) + slots - 1) / slots;
+    const double turns = double(rounds) * slots * FT * (zc + 1.2);
+    return turns <= (is16<T>() ? 1.4 : 1.6) * double(P.n) ? zc : 0;
+}
 
 }  // namespace lbm
 
@@ -1807,14 +1823,14 @@ struct Launchers {
         // as in reduce(); a slab's planes end beside ghost planes, and 16-bit storage is faster in
         // two passes (384^3 FP16: 2.24 against 2.92 ms)
         if constexpr (FLOW && LAT == LAT_D3Q7 && std::is_same<T, float>::value) {
-            if (P.n >= kMarchNodes && P.z_lo == 0 && P.z_hi == P.nz && P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z) {
-                const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
+            if (P.z_lo == 0 && P.z_hi == P.nz && P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z) {
+                int zc = 0;
                 LBM_MODE_SWITCH(mode, {
                     const int nb = resident_blocks(fields_march_kernel<T, M>, 152 * 8);
-                    const int zc = march_chunk(tiles, P.nz, nb, 0.7);
-                    fields_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, out, zc);
+                    zc = march_planes<T>(P, nb);
+                    if (zc) fields_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, out, zc);
                 });
-                return;
+                if (zc) return;
             }
         }
         int bx; const dim3 grid = node_grid(P, bx);
@@ -1846,18 +1862,19 @@ struct Launchers {
         // a whole flow lattice with D3Q7 sets and FP32 arithmetic (a slab, which has no bit field,
         // keeps the neighbours' phi in the phi field; FP64 halos would cost the FP64 pipe)
         if constexpr (FLOW && LAT == LAT_D3Q7 && sizeof(R) == 4) {
-            if (bits && P.n >= kMarchNodes) {
-                int nb = nblocks;
-                const long long tiles = (long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY);
+            if (bits) {
+                int nb = nblocks, zc = 0;
                 LBM_MODE_SWITCH(mode, {
                     nb = resident_blocks(reduce_march_kernel<T, M>, nblocks);
-                    const int zc = march_chunk(tiles, P.nz, nb, 0.7);
-                    reduce_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, partials, zc);
+                    zc = march_planes<T>(P, nb);
+                    if (zc) reduce_march_kernel<T, M><<<nb, dim3(FX, FY), 0, s>>>(P, st, partials, zc);
                 });
-                if (nb < nblocks)
-                    cudaMemsetAsync(partials + (size_t)nb * LBM_NRED_DEV, 0,
-                                    (size_t)(nblocks - nb) * LBM_NRED_DEV * sizeof(double), s);
-                return;
+                if (zc) {
+                    if (nb < nblocks)
+                        cudaMemsetAsync(partials + (size_t)nb * LBM_NRED_DEV, 0,
+                                        (size_t)(nblocks - nb) * LBM_NRED_DEV * sizeof(double), s);
+                    return;
+                }
             }
         }
         if constexpr (FLOW || kTwoD<LAT>) {

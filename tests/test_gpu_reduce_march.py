@@ -16,9 +16,10 @@ from workloads.params import LBMParams
 
 pytestmark = pytest.mark.gpu
 
-# from 600,000 nodes on the lattice is read by the marching kernels, below in separate passes
-SHAPES = [(33, 9, 37), (40, 1, 6), (70, 30, 1), (96, 80, 80), (33, 135, 137), (1, 801, 750), (800, 1, 751),
-          (801, 750, 1)]
+# (96, 80, 80) and the shapes after it are read by the marching kernels (FP32 and 16 bits but the
+# last, FP32), those before it, small, thin or flat, in separate passes
+SHAPES = [(33, 9, 37), (40, 1, 6), (70, 30, 1), (33, 135, 137), (1, 801, 750), (800, 1, 751), (801, 750, 1),
+          (96, 80, 80), (125, 101, 61), (126, 94, 67), (1213, 510, 3)]
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
