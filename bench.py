@@ -3,8 +3,9 @@
 Workload: 512^3 lattice, D3Q19 flow + D3Q7 phi, c^A, c^B, FP32 population storage,
 half-way bounce-back walls at the z ends, periodic in x and y, seeded droplets at
 volume fraction 0.2 with radii in [6, 16] (seed 3). One "step" is one coupled time
-step of the whole lattice: one launch of the fused collide-and-stream kernel, which
-computes the capillary stencil's phi itself. The state (two copies of 21.5 GB) is far
+step of the whole lattice. With FP32 storage that is a small pass for phi of the nodes at
+the x and y ends and one collide-and-stream kernel (loads staged by TMA) that computes the
+other phi of the capillary stencil itself. The state (two copies of 21.5 GB) is far
 larger than the 129 MB L2, so no flush is needed between timed steps.
 
 Prints one JSON line. --impl reference times the FP64 CPU oracle instead (the
@@ -29,10 +30,10 @@ N = 512
 # bytes each node reads and writes per step: 40 populations; 16-bit storage keeps the
 # four rest populations g_0, h^A_0, h^B_0, f_0 in FP32 (36 x 2 B + 4 x 4 B = 88 B each way)
 ALG_BYTES_PER_NODE = {"f32": 320.0, "f16": 176.0, "bf16": 176.0, "f64": 640.0}
-# DRAM bytes (read + write) per node of one fused_flow_kernel<float> launch, from an ncu capture
-# of this kernel at 192^3; traffic scales with the
-# node count. Set to None whenever the kernel changes until it is captured again.
-NCU_DRAM_BYTES_PER_NODE_F32 = 164.05 + 153.90
+# DRAM bytes (read + write) per node of one FP32 step, from an ncu capture at 320^3:
+# flow_tma_kernel 189.6 + 158.7, rim_phi_kernel 15.3 + 0.15 (of the x and y ends: 320/512 of
+# it at 512^3). Set to None whenever the kernels change until they are captured again.
+NCU_DRAM_BYTES_PER_NODE_F32 = 189.6 + 158.7 + 15.4 * 320 / 512
 
 
 def parse():
@@ -176,9 +177,11 @@ def cpu_baseline(init_fields, p, planes, steps):
             "host": host_info()}
 
 
-def time_device(sim, steps, warmup, dist):
+def time_device(sim, steps, warmup, dist, per_kernel=True):
     """Device-timed K steps with CUDA events on the simulation's stream, plus per-kernel
-    event timing of the same region from the library."""
+    event timing of the same region from the library. Steps that go two to a pass are not
+    taken that way while kernels are timed: ``per_kernel`` False leaves them as a user's run
+    has them (and the two kernel times None)."""
     import torch
     sim.step(warmup)
     torch.cuda.synchronize()
@@ -187,15 +190,19 @@ def time_device(sim, steps, warmup, dist):
     torch.cuda.synchronize()
     start = torch.cuda.Event(enable_timing=True)
     stop = torch.cuda.Event(enable_timing=True)
-    sim.profile_begin(steps)
+    if per_kernel:
+        sim.profile_begin(steps)
     start.record(sim.stream)
     sim.step(steps)
     stop.record(sim.stream)
     torch.cuda.synchronize()
     ms = start.elapsed_time(stop)
-    ms_phi, ms_step, nprof = sim.profile_end()
+    if per_kernel:
+        ms_phi, ms_step, nprof = sim.profile_end()
     if dist:
         ms = max_over_ranks(ms, dist, "cuda")
+    if not per_kernel:
+        return ms, None, None
     return ms, ms_phi / max(nprof, 1), ms_step / max(nprof, 1)
 
 
@@ -319,8 +326,10 @@ def gb300(args):
                      "frac": achieved / peak,
                      "traffic": (None if NCU_DRAM_BYTES_PER_NODE_F32 is None or args.storage != "f32"
                                  else NCU_DRAM_BYTES_PER_NODE_F32 * nodes),
-                     "kernel": f"fused_flow_kernel<{'float' if args.storage == 'f32' else args.storage}, BGK> "
-                               "(z-marching fused phi + collide + stream)",
+                     "kernel": {"f32": "rim_phi_kernel + flow_tma_kernel<BGK> (z-marching fused phi + collide + "
+                                       "stream, loads by TMA; below 30 M nodes fused_flow_kernel)",
+                                "bf16": "fused_flow_kernel<bf16, BGK> (z-marching fused phi + collide + stream)"}
+                     .get(args.storage, f"step_kernel<{args.storage}, pull> after phi_kernel"),
                      "alg_bytes_per_launch": bytes_step, "ms_per_launch": ms_step,
                      "peak_kind": f"{peak_kind} hbm_gbs (burst copy)",
                      "whole_step_frac": bytes_step / (ms / args.steps / 1e3) / 1e9 / peak,
@@ -337,27 +346,27 @@ def gb300(args):
         for storage in ("f16", "bf16"):
             q = p.with_(storage=storage)
             v = Simulation(q, *init, device=device)
-            vms, _, vstep = time_device(v, max(20, args.steps // 2), args.warmup, dist)
+            vms, _, _ = time_device(v, max(20, args.steps // 2), args.warmup, dist)
             vs = max(20, args.steps // 2)
             vb = ALG_BYTES_PER_NODE[storage] * nodes
             var[storage] = {"value": ws * nodes * vs / (vms / 1e3) / 1e6, "unit": "MLUPS",
                             "ms_per_step": vms / vs, "speedup_vs_f32": (ms / args.steps) / (vms / vs),
                             "alg_bytes_per_node": ALG_BYTES_PER_NODE[storage],
-                            "roofline_frac": vb / (vstep / 1e3) / 1e9 / peak}
+                            "roofline_frac": vb / (vms / vs / 1e3) / 1e9 / peak}
             del v
             torch.cuda.synchronize()
         # the two-relaxation-time flow collision on the same workload, FP32 storage
         q = p.with_(collision="TRT")
         v = Simulation(q, *init, device=device)
         vs = max(20, args.steps // 2)
-        vms, _, vstep = time_device(v, vs, args.warmup, dist)
+        vms, _, _ = time_device(v, vs, args.warmup, dist)
         var["trt"] = {"value": ws * nodes * vs / (vms / 1e3) / 1e6, "unit": "MLUPS", "ms_per_step": vms / vs,
                       "speedup_vs_f32": (ms / args.steps) / (vms / vs), "collision": "TRT, Lambda = 3/16",
-                      "roofline_frac": ALG_BYTES_PER_NODE["f32"] * nodes / (vstep / 1e3) / 1e9 / peak}
+                      "roofline_frac": ALG_BYTES_PER_NODE["f32"] * nodes / (vms / vs / 1e3) / 1e9 / peak}
         del v
         torch.cuda.synchronize()
-        # the in-place layout (one AA-pattern copy: half the memory of the two-buffer fused
-        # kernel), FP32: a phi pass, then the per-node AA step reading phi from it
+        # the in-place layout (one AA-pattern copy: half the memory of the two-buffer
+        # layout), FP32: a phi pass, then the per-node AA step reading phi from it
         q = p.with_(inplace=True)
         v = Simulation(q, *init, device=device)
         vs = max(20, args.steps // 2)
@@ -386,10 +395,10 @@ def gb300(args):
         q = p.with_(collision="MRT")
         v = Simulation(q, *init, device=device)
         vs = max(20, args.steps // 2)
-        vms, _, vstep = time_device(v, vs, args.warmup, dist)
+        vms, _, _ = time_device(v, vs, args.warmup, dist)
         var["mrt"] = {"value": ws * nodes * vs / (vms / 1e3) / 1e6, "unit": "MLUPS", "ms_per_step": vms / vs,
                       "speedup_vs_f32": (ms / args.steps) / (vms / vs), "collision": "MRT, d'Humieres rates",
-                      "roofline_frac": ALG_BYTES_PER_NODE["f32"] * nodes / (vstep / 1e3) / 1e9 / peak}
+                      "roofline_frac": ALG_BYTES_PER_NODE["f32"] * nodes / (vms / vs / 1e3) / 1e9 / peak}
         del v
         torch.cuda.synchronize()
         # D3Q19 for phi, c^A, c^B (the paper's lattice for every equation): 76 populations,
@@ -404,35 +413,37 @@ def gb300(args):
                                 "roofline_frac": b19 * nodes / (vms / vs / 1e3) / 1e9 / peak}
         del v
         torch.cuda.synchronize()
-        # 3D ripening without flow (256^3, D3Q7, FP32, in place): 21 populations, 168 B/node
+        # 3D ripening without flow (256^3, D3Q7, FP32): 21 populations, 168 B/node a pass of two steps
         from workloads import configs
         p3, f3 = configs.ripening()
         v = Simulation(p3, *f3(device=device), device=device)
         vs = max(20, args.steps // 2)
-        vms, _, _ = time_device(v, vs, args.warmup, dist)
+        vs -= vs % 4
+        vms, _, _ = time_device(v, vs, args.warmup - args.warmup % 2, dist, per_kernel=False)
         s3 = v.sums()
-        b3 = 2 * 21 * 4.0
+        b3 = 2 * 21 * 4.0 / 2
         var["ripening_3d"] = {"value": ws * p3.nodes * vs / (vms / 1e3) / 1e6, "unit": "MLUPS",
-                              "ms_per_step": vms / vs, "workload": "256^3 D3Q7, no flow, fraction 0.15, FP32, in place",
+                              "ms_per_step": vms / vs, "workload": "256^3 D3Q7, no flow, fraction 0.15, FP32, two steps a pass",
                               "alg_bytes_per_node": b3, "roofline_frac": b3 * p3.nodes / (vms / vs / 1e3) / 1e9 / peak,
-                              "droplets_N": s3["euler"], "after_steps": args.warmup + vs}
+                              "droplets_N": s3["euler"], "after_steps": v.t}
         del v
         torch.cuda.synchronize()
-        # 2D ripening without flow on D2Q9 (§4.2.2 table): 4096^2, 27 FP32 populations in place,
+        # 2D ripening without flow on D2Q9 (§4.2.2 table): 4096^2, 27 FP32 populations, two steps a pass,
         # with the one-pass droplet count and mean radius of Eq. 67 after the timed steps
         from workloads import configs
         p2, f2 = configs.ripening_2d()
         v = Simulation(p2, *f2(device=device), device=device)
         vs = max(20, args.steps // 2)
-        vms, _, _ = time_device(v, vs, args.warmup, dist)
+        vs -= vs % 4
+        vms, _, _ = time_device(v, vs, args.warmup - args.warmup % 2, dist, per_kernel=False)
         s2 = v.sums()
-        b2 = 2 * 27 * 4.0
+        b2 = 2 * 27 * 4.0 / 2
         n2 = p2.nodes
         var["ripening_2d"] = {"value": ws * n2 * vs / (vms / 1e3) / 1e6, "unit": "MLUPS", "ms_per_step": vms / vs,
-                              "workload": "4096^2 D2Q9, no flow, phase fraction 0.08, FP32, in place",
+                              "workload": "4096^2 D2Q9, no flow, phase fraction 0.08, FP32, two steps a pass",
                               "alg_bytes_per_node": b2, "roofline_frac": b2 * n2 / (vms / vs / 1e3) / 1e9 / peak,
                               "droplets_N": s2["euler"], "mean_radius": s2["interface"] / (2 * math.pi * s2["euler"]),
-                              "after_steps": args.warmup + vs}
+                              "after_steps": v.t}
         del v
         torch.cuda.synchronize()
         out["variants"] = var

@@ -11,7 +11,8 @@
  * D3Q19 with a BGK, TRT or MRT collision.
  * One call of lbm_step advances every population set by one fused collide-and-stream
  * pass over HBM: in-place AA-pattern streaming without flow; with flow, by default, a
- * two-buffer pull step that computes the capillary stencil's phi on the fly.
+ * two-buffer pull step that computes the capillary stencil's phi on the fly or, where that is
+ * faster (LBM_F16, LBM_F64, small LBM_F32 lattices), reads it from a phi pass.
  *
  * Memory: every device buffer is allocated and owned by the caller (for instance a
  * torch tensor); the library never allocates or frees device memory. The context is
@@ -82,8 +83,8 @@ typedef struct lbm_params {
     int32_t wall_x;          /* 1: half-way bounce-back planes at x = -1/2 and nx - 1/2 */
     int32_t wall_z;          /* 1: half-way bounce-back planes at z = -1/2 and nz - 1/2 */
     int32_t source_off;      /* 1: S_phi = 0 (pure advection-diffusion of phi; test switch) */
-    int32_t inplace;         /* flow only. 0: two state copies, one fused kernel per step (the
-                              * capillary stencil's phi is computed on the fly in shared memory);
+    int32_t inplace;         /* flow only. 0: two state copies, a pull step (the capillary stencil's
+                              * phi computed on the fly in shared memory, or by a phi pass);
                               * 1: one in-place AA-pattern copy (half the memory) plus a phi pass.
                               * Without flow the state is always one in-place AA-pattern copy. */
     double W;                /* interface width (Eq. 14) */
@@ -161,8 +162,10 @@ lbm_status lbm_attach(const lbm_params* p, void* d_state, void* d_work, int64_t 
                       void* stream, lbm_ctx** out);
 
 /* Advance nsteps >= 0 coupled time steps (§3): one fused collide-and-stream kernel per
- * step; with flow, the in-place layout and the LBM_D3Q19 scalar lattice add a phi pass for
- * the capillary stencil (lbm_kernels_per_step). Asynchronous. */
+ * step; with flow, all but LBM_BF16 and FP32 lattices of 600,000 nodes and more with two copies
+ * and LBM_D3Q7 scalars add a phi pass for the capillary stencil, and FP32 lattices of 30
+ * million nodes and more a pass for phi of their x and y ends (lbm_kernels_per_step). The
+ * passes use the phi field of the work buffer. Asynchronous. */
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
 
 /* lbm_step with a scratch buffer: with FP32 storage and no flow (LBM_D3Q7 from a million nodes
@@ -210,8 +213,8 @@ lbm_status lbm_reduce(lbm_ctx* ctx, double* out);
 lbm_status lbm_profile_begin(lbm_ctx* ctx, int max_steps);
 lbm_status lbm_profile_end(lbm_ctx* ctx, double* out);
 
-/* Number of kernels one lbm_step(ctx, 1) launches: 2 with flow unless the state has two
- * copies and the scalar lattice is LBM_D3Q7 (the fused kernel), else 1; 0 for NULL. */
+/* Number of kernels one lbm_step(ctx, 1) launches: 2 with flow where a phi pass or a pass for
+ * phi of the lattice's ends comes first (see lbm_step), else 1; 0 for NULL. */
 int lbm_kernels_per_step(const lbm_ctx* ctx);
 
 /* One step (§3) out of place, without a context: d_src holds one state copy at time t (the
