@@ -168,8 +168,8 @@ __device__ __forceinline__ void block_accumulate(const R* acc, double* __restric
 // Grid as the forward step: x along threads, y and z along blocks; one node per thread.
 template <class T, int LAT, int MODE>
 __global__ void __launch_bounds__(kBlockX)
-adjoint_step_kernel(const DevParams P, const StateView st, const typename RealOf<T>::type* __restrict__ lam_next,
-                    typename RealOf<T>::type* __restrict__ lam, double* __restrict__ partials, double om_g_deriv) {
+adjoint_step_kernel(const DevParams P, const StateView st, const typename RealOf<T>::type* lam_next,
+                    typename RealOf<T>::type* lam, double* partials, double om_g_deriv) {
     using R = typename RealOf<T>::type;
     using L = Scalar<LAT>;
     constexpr int Q = L::Q;

@@ -112,7 +112,7 @@ __device__ __forceinline__ void load_box(unsigned to, const CUtensorMap* m, int 
 template <int COLL>
 __global__ void __launch_bounds__(tma::T, 1)
 flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const StateView src, const StateView dst,
-                const float* __restrict__ rim_phi, int zchunk) {
+                const float* rim_phi, int zchunk) {
     using namespace tma;
     constexpr int kColl = COLL == 2 ? 2 : -1;
     extern __shared__ __align__(128) unsigned char tma_smem[];
@@ -386,7 +386,7 @@ flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const
 
 // phi of the nodes at the ends of the lattice in x and y, which tiles at the opposite ends read.
 static __global__ void __launch_bounds__(kBlockX)
-rim_phi_kernel(const DevParams P, const StateView st, float* __restrict__ phi_out) {
+rim_phi_kernel(const DevParams P, const StateView st, float* phi_out) {
     begin_after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.z;
     const int rows = 2 * P.nx, c = i - rows;

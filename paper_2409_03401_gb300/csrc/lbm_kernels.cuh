@@ -23,6 +23,9 @@ constexpr int kBlockX = 128;
 // Step kernels follow one another in a stream with programmatic dependent launch: the next
 // one's blocks are set up while the last blocks of this one still run (launch_dependents, once
 // every block has started), and wait there until it has completed and its stores are visible.
+// What an earlier kernel of the stream writes is read through plain pointers: a const __restrict__
+// one allows read-only loads, whose data must not change while the kernel lives, and its blocks
+// may be there before those stores are.
 __device__ __forceinline__ void begin_after_previous() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -128,7 +131,7 @@ struct Addr {
     }
     // phi of a neighbour in a phi array, mirror ghost across walls (zero normal gradient)
     template <class R>
-    __device__ __forceinline__ R phi(const R* __restrict__ f, int dx, int dy, int dz) const {
+    __device__ __forceinline__ R phi(const R* f, int dx, int dy, int dz) const {
         const int xx = nb.c[0][dx + 1] >= 0 ? nb.c[0][dx + 1] : nb.c[0][1];
         const int r = nb.c[2][dz + 1] >= 0 ? nb.row[dz + 1][dy + 1] : nb.row[1][dy + 1];
         return f[r + xx];
@@ -169,7 +172,7 @@ struct AddrInner {
         return k == 0 ? self : beside(-ex, -ey, -ez);
     }
     template <class R>
-    __device__ __forceinline__ R phi(const R* __restrict__ f, int dx, int dy, int dz) const {
+    __device__ __forceinline__ R phi(const R* f, int dx, int dy, int dz) const {
         return f[beside(dx, dy, dz)];
     }
 };
@@ -759,7 +762,7 @@ __device__ __forceinline__ void collide_store(const Node<T, LAT, FLOW>& nd, type
 // The step of one node at address ``ad``.
 template <class T, int LAT, bool FLOW, int COLL, class A>
 __device__ __forceinline__ void step_node(const A& ad, const DevParams& P, const StateView& st, const StateView& out,
-                                          const typename RealOf<T>::type* __restrict__ phi_field) {
+                                          const typename RealOf<T>::type* phi_field) {
     using R = typename RealOf<T>::type;
     Node<T, LAT, FLOW> nd;
     nd.gather(st, ad, P);
@@ -783,8 +786,7 @@ __device__ __forceinline__ void step_node(const A& ad, const DevParams& P, const
 // phi_field (phi pass); MODE AA_* works in place on ``st``, PULL reads ``st`` and writes ``out``.
 template <class T, int LAT, bool FLOW, int MODE, int COLL>
 __global__ void __launch_bounds__(kBlockX)
-step_kernel(const DevParams P, const StateView st, const StateView out,
-            const typename RealOf<T>::type* __restrict__ phi_field) {
+step_kernel(const DevParams P, const StateView st, const StateView out, const typename RealOf<T>::type* phi_field) {
     using R = typename RealOf<T>::type;
     begin_after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -815,7 +817,7 @@ constexpr long long kAfterBlocks = 8192;
 // AFTER: launched after a step kernel with launch_after_previous.
 template <class T, int LAT, int MODE, bool AFTER>
 __global__ void __launch_bounds__(kBlockX)
-phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* __restrict__ phi_out) {
+phi_kernel(const DevParams P, const StateView st, typename RealOf<T>::type* phi_out) {
     if constexpr (AFTER) begin_after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + P.z_lo;
