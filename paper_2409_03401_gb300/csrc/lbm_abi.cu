@@ -187,6 +187,7 @@ struct lbm_ctx {
     std::vector<cudaEvent_t> ev;   // profiling: 3 events per timed step
     int prof_max = 0, prof_n = 0;
     cudaGraphExec_t graph = nullptr;   // two steps captured from an even time level
+    bool waits = false;            // kernels with bounded waits were queued (the fault word is in use)
     // slab of a z-decomposed lattice (lbm_slab_init): global first plane, own planes, and
     // whether a neighbour's plane sits below / above (ghost planes z_lo - 1 and z_hi)
     bool slab = false;
@@ -356,6 +357,19 @@ void ghost_phi_to_field(lbm_ctx* c) {
                                 cudaMemcpyDeviceToDevice, c->stream);
 }
 
+// The word that a kernel whose bounded wait ran out sets: behind the sums of lbm_reduce, which
+// reads it. Cleared before the first such kernel of a context.
+unsigned* fault_of(const lbm_ctx* c) {
+    return reinterpret_cast<unsigned*>(c->work + c->L.off_out + LBM_NRED * sizeof(double));
+}
+void clear_fault_once(lbm_ctx* c) {
+    if (!c->waits) cudaMemsetAsync(fault_of(c), 0, sizeof(double), c->stream);
+    c->waits = true;
+}
+bool tma_step(const lbm_ctx* c) {
+    return one_pass(c) && c->p.storage == LBM_F32 && !c->slab && lbm::flow_tma_applies(c->dp);
+}
+
 // Queue the kernels that advance time level t to t + 1 (no change to the context).
 void launch_one(lbm_ctx* c, int64_t t, cudaEvent_t* e) {
     const int mode = c->L.two ? lbm::kModePull : ((t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven);
@@ -370,7 +384,8 @@ void launch_one(lbm_ctx* c, int64_t t, cudaEvent_t* e) {
     }
     if (e) cudaEventRecord(e[1], c->stream);
     if (fused) {
-        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, c->slab ? nullptr : c->work + c->L.off_phi, c->stream);
+        LBM_DISPATCH(c->p.storage, launch_fused, c->dp, src, dst, c->slab ? nullptr : c->work + c->L.off_phi, fault_of(c),
+                     c->stream);
     } else {
         LBM_DISPATCH(c->p.storage, launch_step, c->dp, src, dst, c->p.lattice, c->p.flow != 0, mode,
                      c->work + c->L.off_phi, c->stream);
@@ -385,6 +400,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     if (c->slab && nsteps > 1)
         return fail(c, LBM_ERR_STATE, "a slab advances one step per call: exchange its halos between steps");
     cudaGetLastError();
+    if (nsteps > 0 && tma_step(c)) clear_fault_once(c);
     for (int i = 0; i < nsteps; ++i) {
         const bool timed = c->prof_n < c->prof_max;
         launch_one(c, c->t, timed ? &c->ev[3 * c->prof_n] : nullptr);
@@ -414,9 +430,10 @@ lbm_status lbm_step_scratch(lbm_ctx* c, int nsteps, void* d_scratch, size_t scra
     }
     const StateView mid = view_of(&c->p, c->L, d_scratch);
     cudaGetLastError();
+    if (nsteps >= 4) clear_fault_once(c);
     for (; nsteps >= 4; nsteps -= 4) {                // there and back: the state ends in its own buffer
-        LBM_DISPATCH(c->p.storage, launch_two_steps, c->dp, c->st, mid, c->p.lattice, c->stream);
-        LBM_DISPATCH(c->p.storage, launch_two_steps, c->dp, mid, c->st, c->p.lattice, c->stream);
+        LBM_DISPATCH(c->p.storage, launch_two_steps, c->dp, c->st, mid, c->p.lattice, fault_of(c), c->stream);
+        LBM_DISPATCH(c->p.storage, launch_two_steps, c->dp, mid, c->st, c->p.lattice, fault_of(c), c->stream);
         c->t += 4;
     }
     lbm_status s = cuda_check(c, "two-step kernel launch");
@@ -500,8 +517,7 @@ lbm_status lbm_profile_end(lbm_ctx* c, double* out) {
 
 int lbm_kernels_per_step(const lbm_ctx* c) {
     if (!c) return 0;
-    const bool rim_pass = one_pass(c) && c->p.storage == LBM_F32 && !c->slab && lbm::flow_tma_applies(c->dp);
-    return (c->p.flow && !one_pass(c)) || rim_pass ? 2 : 1;
+    return (c->p.flow && !one_pass(c)) || tma_step(c) ? 2 : 1;
 }
 
 int64_t lbm_time(const lbm_ctx* c) { return c ? c->t : -1; }
@@ -532,9 +548,15 @@ lbm_status lbm_reduce(lbm_ctx* c, double* out) {
     reduce_final<<<1, 256, 0, c->stream>>>(partials, kRedBlocks, dout);
     lbm_status s = cuda_check(c, "reduce kernel launch");
     if (s != LBM_OK) return s;
-    cudaError_t e = cudaMemcpyAsync(out, dout, LBM_NRED * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    double host[LBM_NRED + 1];                         // the sums, and the fault word behind them
+    cudaError_t e = cudaMemcpyAsync(host, dout, sizeof host, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return fail(c, LBM_ERR_CUDA, std::string("reduce copy: ") + cudaGetErrorString(e));
+    std::memcpy(out, host, LBM_NRED * sizeof(double));
+    unsigned fault;
+    std::memcpy(&fault, host + LBM_NRED, sizeof fault);
+    if (c->waits && fault == lbm::kWaitFault)
+        return fail(c, LBM_ERR_CUDA, "a wait in a step kernel ran out: the state is not valid");
     if (out[LBM_RED_NONFINITE] != 0.0)
         return fail(c, LBM_ERR_UNSTABLE, "non-finite moments in the state (unstable run)");
     return LBM_OK;
@@ -558,7 +580,7 @@ lbm_status lbm_step_buffers(const lbm_params* p, const void* d_src, void* d_dst,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaGetLastError();
     if (L.two && fused_flow(p)) {
-        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, nullptr, s);
+        LBM_DISPATCH(p->storage, launch_fused, dp, src, dst, nullptr, nullptr, s);
     } else {
         const int mode = L.two ? lbm::kModePull : ((t & 1) ? lbm::kModeAAOdd : lbm::kModeAAEven);
         char* phi = static_cast<char*>(d_work) + L.off_phi;

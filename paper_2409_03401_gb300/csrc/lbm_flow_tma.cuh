@@ -112,7 +112,7 @@ __device__ __forceinline__ void load_box(unsigned to, const CUtensorMap* m, int 
 template <int COLL>
 __global__ void __launch_bounds__(tma::T, 1)
 flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const StateView src, const StateView dst,
-                const float* rim_phi, int zchunk) {
+                const float* rim_phi, unsigned* fault, int zchunk) {
     using namespace tma;
     constexpr int kColl = COLL == 2 ? 2 : -1;
     extern __shared__ __align__(128) unsigned char tma_smem[];
@@ -198,11 +198,25 @@ flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const
     }
     const int hx = x0 - 1 + hj, hy = y0 - 1 + hi;
 
-    // ``ok``: every copy so far arrived. Once one did not (a wait ran out), the block goes on
-    // without waiting, its barriers matched, and marks its nodes as not finite.
+    // ``ok``: every copy so far arrived, for the whole block from the next __syncthreads_and on.
     bool ok = true;
     auto wait = [&](unsigned b, unsigned parity) { if (ok) ok = bar_wait(b, parity & 1); };
-    auto wait_scalars = [&](int zz, int slot) { wait(bars + 8 * slot, unsigned(zz - (zs - 1)) / 3); };
+    auto scalars_phase = [&](int zz) { return unsigned(zz - (zs - 1)) / 3; };
+    auto wait_scalars = [&](int zz, int slot) { wait(bars + 8 * slot, scalars_phase(zz)); };
+    // A wait ran out before plane z was collided: no more copies, those in flight (scalars up to
+    // plane ``last``, the flow of plane z) land or are waited for once more, before the block's
+    // shared memory goes to another; the fault word is set, and the planes the block has not
+    // written are marked as not finite.
+    auto give_up = [&](int z, int last) {
+        for (int zz = max(last - 2, zs - 1); zz <= last; ++zz)
+            bar_wait(bars + 8 * ((zz - (zs - 1)) % 3), scalars_phase(zz) & 1);
+        bar_wait(bars + 24, unsigned(z - zs) & 1);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (tid == 0) *fault = kWaitFault;
+        if (active)
+            for (int zz = z; zz < ze; ++zz)
+                static_cast<float*>(dst.plane[Planes<LAT_D3Q7>::HA])[node_of(x, y, zz, P)] = __int_as_float(0x7fc00000);
+    };
 
     // Tiles whose sources reach past the lattice's end in x or y, where the copies leave zeros: the
     // threads fetch the wrapped values themselves, most of a plane's time ahead like the copies (a
@@ -309,7 +323,8 @@ flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const
     wait_scalars(zs - 1, 0);
     fill_own(zs - 1, 0);
     fill_halo(zs - 1, 0);
-    __syncthreads();                                                   // slot 0 is free again
+    ok = __syncthreads_and(ok);                                        // slot 0 is free again
+    if (!ok) return give_up(zs, zs + 1);
     if (zs + 1 < ze) load_scalars(zs + 2, 0);
     if (edge) {
         if (zs + 1 < ze) fetch_scalars(zs + 2);
@@ -351,7 +366,9 @@ flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const
                 if (ey_m) nd.f[ym[i]] = ends.f_y[i][tx];
             }
         }
-        __syncthreads();                       // phi of plane z + 1 is there; slot and flow are read no more
+        // phi of plane z + 1 is there; slot and flow are read no more
+        ok = __syncthreads_and(ok);
+        if (!ok) return give_up(z, z + 1 < ze ? z + 2 : z + 1);
         // the flow first: it is wanted in a plane's time, the scalars in two (8.6 ms a step at 512^3
         // the other way round)
         if (z + 1 < ze) load_flow(z + 1);
@@ -376,7 +393,6 @@ flow_tma_kernel(const DevParams P, const __grid_constant__ tma::Maps maps, const
                         return ring[dz < 0 ? sp : (dz > 0 ? sn : sc)][ty + 1 + dy][tx + 1 + dx];
                     }, phi, gx, gy, gz, lap);
             force_velocity(nd, phi, gx, gy, gz, lap, P, Fx, Fy, Fz, ux, uy, uz);
-            if (!ok) nd.dcA = __int_as_float(0x7fc00000);              // a copy that never came: the state shows it
             collide_store<float, LAT_D3Q7, true, AddrInterior, kColl>(nd, phi, ux, uy, uz, Fx, Fy, Fz, dst,
                                                                       AddrInterior{self, P.nx, P.nx * P.ny}, P);
         }

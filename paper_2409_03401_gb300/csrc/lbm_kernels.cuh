@@ -1752,11 +1752,12 @@ struct Launchers {
         LBM_MODE_SWITCH(mode, launch_after_previous<R>(step_kernel<T, LAT, FLOW, M, -1>, grid, dim3(bx), 0, s, P, st, out, phi));
     }
     template <int LAT>
-    static void two_steps(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
-        launch_two_steps_at<T, LAT>(P, src, dst, s);
+    static void two_steps(const DevParams& P, const StateView& src, const StateView& dst, unsigned* fault, cudaStream_t s) {
+        launch_two_steps_at<T, LAT>(P, src, dst, fault, s);
     }
     template <int COLL>
-    static bool flow_tma(const DevParams& P, const StateView& src, const StateView& dst, R* phi, cudaStream_t s) {
+    static bool flow_tma(const DevParams& P, const StateView& src, const StateView& dst, R* phi, unsigned* fault,
+                         cudaStream_t s) {
         if constexpr (std::is_same<T, float>::value) {
             tma::Maps maps;
             if (!tma_maps(P, src, maps)) return false;
@@ -1771,16 +1772,18 @@ struct Launchers {
             launch_after_previous<R>(rim_phi_kernel, dim3((2 * (P.nx + P.ny - 2) + kBlockX - 1) / kBlockX, 1, P.nz),
                                      dim3(kBlockX), 0, s, P, src, phi);
             launch_after_previous<R>(flow_tma_kernel<COLL>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(tma::T),
-                                     size_t(tma::kSmem), s, P, maps, src, dst, phi, zc);
+                                     size_t(tma::kSmem), s, P, maps, src, dst, phi, fault, zc);
             return true;
         }
         return false;
     }
-    // ``phi_work``: a phi field to use as scratch, or nullptr
-    static void fused(const DevParams& P, const StateView& src, const StateView& dst, void* phi_work, cudaStream_t s) {
+    // ``phi_work``: a phi field to use as scratch, or nullptr; with one, ``fault``: the word that a
+    // wait that ran out sets to kWaitFault
+    static void fused(const DevParams& P, const StateView& src, const StateView& dst, void* phi_work, unsigned* fault,
+                      cudaStream_t s) {
         if (std::is_same<T, float>::value && phi_work && flow_tma_applies(P)) {
             R* phi = static_cast<R*>(phi_work);
-            if (P.coll == 2 ? flow_tma<2>(P, src, dst, phi, s) : flow_tma<0>(P, src, dst, phi, s)) return;
+            if (P.coll == 2 ? flow_tma<2>(P, src, dst, phi, fault, s) : flow_tma<0>(P, src, dst, phi, fault, s)) return;
         }
         const dim3 block(FX, FY);
         const int zchunk = march_chunk((long long)((P.nx + FX - 1) / FX) * ((P.ny + FY - 1) / FY), P.z_hi - P.z_lo,
@@ -1932,16 +1935,16 @@ struct Launchers {
         else Launchers<T>::step<LAT_D3Q7, false>(P, st, out, mode, phi, s);                                \
     }                                                                                                     \
     void launch_two_steps_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst, int lat, \
-                                   cudaStream_t s) {                                                      \
+                                   unsigned* fault, cudaStream_t s) {                                     \
         if constexpr (sizeof(T) == 4) {                                                                   \
-            if (lat == LAT_D2Q5) Launchers<T>::two_steps<LAT_D2Q5>(P, src, dst, s);                        \
-            else if (lat == LAT_D2Q9) Launchers<T>::two_steps<LAT_D2Q9>(P, src, dst, s);                   \
-            else Launchers<T>::two_steps<LAT_D3Q7>(P, src, dst, s);                                       \
+            if (lat == LAT_D2Q5) Launchers<T>::two_steps<LAT_D2Q5>(P, src, dst, fault, s);                 \
+            else if (lat == LAT_D2Q9) Launchers<T>::two_steps<LAT_D2Q9>(P, src, dst, fault, s);            \
+            else Launchers<T>::two_steps<LAT_D3Q7>(P, src, dst, fault, s);                                \
         }                                                                                                 \
     }                                                                                                     \
     void launch_fused_##SUFFIX(const DevParams& P, const StateView& src, const StateView& dst,            \
-                               void* phi_work, cudaStream_t s) {                                          \
-        Launchers<T>::fused(P, src, dst, phi_work, s);                                                    \
+                               void* phi_work, unsigned* fault, cudaStream_t s) {                         \
+        Launchers<T>::fused(P, src, dst, phi_work, fault, s);                                             \
     }                                                                                                     \
     void launch_fields_##SUFFIX(const DevParams& P, const StateView& st, int lat, bool flow, int mode,    \
                                 void* phi, FieldPtrs out, cudaStream_t s) {                               \

@@ -16,6 +16,9 @@ struct FieldPtrs { void* p[LBM_NFIELDS_DEV]; };
 // streaming modes (see lbm_kernels.cuh)
 constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
 
+// What a kernel whose bounded wait ran out leaves in the context's fault word.
+constexpr unsigned kWaitFault = 0x57414954u;
+
 // Whether an FP32 two-buffer flow step on D3Q7 sets takes the TMA-staged kernel (given a phi field
 // as scratch): rows of whole 16-byte pieces (a tensor copy's rule), the undivided lattice, no
 // walls in x, and 30 million nodes, so that the tiles at the lattice's ends are few enough for
@@ -36,9 +39,9 @@ inline bool flow_tma_applies(const DevParams& P) {
     void launch_step_##SUFFIX(const DevParams&, const StateView&, const StateView&, int lat, bool flow, \
                               int mode, void* phi, cudaStream_t);                                        \
     void launch_two_steps_##SUFFIX(const DevParams&, const StateView&, const StateView&, int lat,        \
-                                   cudaStream_t);                                                         \
+                                   unsigned* fault, cudaStream_t);                                        \
     void launch_fused_##SUFFIX(const DevParams&, const StateView&, const StateView&, void* phi_work,      \
-                               cudaStream_t);                                                            \
+                               unsigned* fault, cudaStream_t);                                           \
     void launch_fields_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, int mode,        \
                                 void* phi, FieldPtrs, cudaStream_t);                                     \
     void launch_reduce_##SUFFIX(const DevParams&, const StateView&, int lat, bool flow, int mode,        \

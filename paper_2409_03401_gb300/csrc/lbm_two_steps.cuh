@@ -109,7 +109,7 @@ constexpr int kTwoStepsBlocks = 2;
 
 template <class T>
 __global__ void __launch_bounds__(T2X * T2Y, kTwoStepsBlocks)
-two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst, int zchunk) {
+two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst, unsigned* fault, int zchunk) {
     begin_after_previous();
     using R = typename RealOf<T>::type;
     constexpr int Q = 7;
@@ -184,7 +184,7 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
                 in[s][4] = ys[slot][2 * s + 1][ty + 1][tx];
                 in[s][6] = top ? up[s] : o[s][6];
             }
-            if (!ok) in[1][0] = __int_as_float(0x7fc00000);            // never in a run: the state shows it
+            if (!ok) in[1][0] = __int_as_float(0x7fc00000);            // the wait ran out: the state shows it
             const int zp = z + 1 == P.nz ? 0 : z + 1, zm = z == 0 ? P.nz - 1 : z - 1;
             const int self = z * nxy + col;
             collide_second<T, LAT_D3Q7>(in, dst, self, inner, wall_lo, wall_hi, P, [&](int k) -> Slot {
@@ -205,6 +205,7 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
         }
         slot = next;
     }
+    if (!ok) *fault = kWaitFault;
 }
 
 // 2D: a warp marches along y on its own; its 28 inner lanes own nodes, the two outer ones on each
@@ -284,14 +285,14 @@ two_steps_2d_kernel(const DevParams P, const StateView src, const StateView dst,
 }
 
 template <class T, int LAT>
-void launch_two_steps_at(const DevParams& P, const StateView& src, const StateView& dst, cudaStream_t s) {
+void launch_two_steps_at(const DevParams& P, const StateView& src, const StateView& dst, unsigned* fault, cudaStream_t s) {
     if constexpr (LAT == LAT_D3Q7) {
         const dim3 tiles((P.nx + T2IX - 1) / T2IX, (P.ny + T2IY - 1) / T2IY);
         const int zc = march_chunk((long long)tiles.x * tiles.y, P.nz, 152 * kTwoStepsBlocks, 2.0);
         constexpr int smem = 4 * 6 * T2Y * T2X * int(sizeof(float)) + 64;
         cudaFuncSetAttribute(two_steps_3d_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         launch_after_previous<float>(two_steps_3d_kernel<T>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(T2X, T2Y),
-                                     size_t(smem), s, P, src, dst, zc);
+                                     size_t(smem), s, P, src, dst, fault, zc);
     } else {
         const int wins = (P.nx + T2IX - 1) / T2IX, bx = (wins + T2Warps - 1) / T2Warps;
         const int yc = march_chunk(bx, P.ny, 152 * kTwoSteps2DBlocks, 2.0);
