@@ -9,8 +9,8 @@
 // registers meanwhile; here 100 KB are in flight whatever the warps do, no load instruction or
 // address is left per population, and nothing is parked. 512^3, a step: 8.19 -> 7.39 ms (0.77 ->
 // 0.86 of the copy bandwidth at 320 B a node); tiles inside the lattice alone run at 0.94, bound
-// by HBM (with every copy left out the rest takes 4.6 ms); the tiles at the lattice's ends in x
-// and y, which the copies do not wrap around, take about twice the time.
+// by HBM (with every copy left out the rest takes 4.6 ms); the tiles at the lattice's ends, which
+// the copies do not wrap around, take 1.4 times as long at an end in x, hardly longer in y.
 #pragma once
 
 #include <cuda.h>

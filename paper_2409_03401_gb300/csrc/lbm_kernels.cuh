@@ -1639,19 +1639,6 @@ fields_march_kernel(const DevParams P, const StateView st, FieldPtrs out, int zc
     });
 }
 
-// Planes (rows, in 2D) a marching block goes through: the count, up to ``most``, for which the
-// waves of blocks over the chip's ``slots`` times the planes each block computes, ``extra`` for
-// the planes around the chunk among them, are fewest.
-inline int march_chunk(long long tiles, int n, long long slots, double extra, int most = 32) {
-    int best = 1;
-    double cost = 1e300;
-    for (int c = 1; c <= n && c <= most; ++c) {
-        const long long blocks = tiles * ((n + c - 1) / c);
-        const double t = double((blocks + slots - 1) / slots) * (c + extra);
-        if (t <= cost) { cost = t; best = c; }
-    }
-    return best;
-}
 // Planes per item of the marching diagnostics and fields on ``slots`` resident blocks, or 0 where
 // separate passes are faster: below kMarchNodes, and where the threads' turns, empty ones of
 // ragged tiles and of the last round among them, are many for each node. Turns a node and the

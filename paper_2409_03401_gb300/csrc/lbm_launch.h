@@ -19,14 +19,36 @@ constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
 // What a kernel whose bounded wait ran out leaves in the context's fault word.
 constexpr unsigned kWaitFault = 0x57414954u;
 
+// Planes (rows, in 2D) a marching block goes through: the count, up to ``most``, for which the
+// waves of blocks over the chip's ``slots`` times the planes each block computes, ``extra`` for
+// the planes around the chunk among them, are fewest.
+inline int march_chunk(long long tiles, int n, long long slots, double extra, int most = 32) {
+    int best = 1;
+    double cost = 1e300;
+    for (int c = 1; c <= n && c <= most; ++c) {
+        const long long blocks = tiles * ((n + c - 1) / c);
+        const double t = double((blocks + slots - 1) / slots) * (c + extra);
+        if (t <= cost) { cost = t; best = c; }
+    }
+    return best;
+}
+
 // Whether an FP32 two-buffer flow step on D3Q7 sets takes the TMA-staged kernel (given a phi field
 // as scratch): rows of whole 16-byte pieces (a tensor copy's rule), the undivided lattice, no
-// walls in x, and 30 million nodes, so that the tiles at the lattice's ends are few enough for
-// what they cost more (512^3: 7.39 against 8.19 ms a step, 384^3: 3.20 against 3.46 ms, 256^3:
-// 1.05 against 1.04 ms, 192^3: 0.49 against 0.44 ms).
+// walls in x, 30 million nodes (measured from there on), and tiles that are
+// worth it: a column of 32 x 15 threads at an end in x takes 1.4 times as long as another. Threads
+// a node weighted so, and the fused kernel's time over this one's: 512^3 1.08, 1.107 (MRT 1.046);
+// 384^3 1.08, 1.060; 2048x128x128 1.07, 1.137 (MRT 1.078); 512x243x242 1.10, 1.082; 552x700x118 MRT
+// 1.10, 1.047; 800x96x400 1.13, 1.070; 224x224x640 1.12, 0.990; 256x256x458 1.16, 0.991 (MRT 0.955);
+// 216x284x741 MRT 1.16, 0.974; 128x2048x128 1.20, 0.907; 128x128x2048 1.27, 0.888; 64x700x671 1.41,
+// 0.789; 1024x32x917 1.44, 0.884. In flat lattices the planes around a chunk weigh more: 2048x2048x8
+// 1.045, 4096x2048x4 1.006 (MRT 0.970), 4096x4096x2 0.985.
 inline bool flow_tma_applies(const DevParams& P) {
-    return P.nx % 4 == 0 && P.nx >= 64 && P.ny >= 32 && P.n >= 30000000 && !P.wall_x && P.z_lo == 0 && P.z_hi == P.nz &&
-           P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z;
+    if (!(P.nx % 4 == 0 && P.nx >= 64 && P.ny >= 32 && P.nz >= 8 && P.n >= 30000000 && !P.wall_x && P.z_lo == 0 &&
+          P.z_hi == P.nz && P.wall_zlo == P.wall_z && P.wall_zhi == P.wall_z))
+        return false;
+    const int tx = (P.nx + 31) / 32, ty = (P.ny + 14) / 15;            // two of the tx columns stand at an end
+    return 32.0 * 15.0 * (tx + 0.4 * 2) * ty <= (P.coll == 2 ? 1.09 : 1.13) * P.nx * P.ny;
 }
 
 #define LBM_DECLARE_LAUNCHERS(SUFFIX)                                                                   \
