@@ -28,11 +28,12 @@ bool fused_flow(const lbm_params* p) { return p->flow && p->lattice == LBM_D3Q7;
 // Lattices stepped two steps per pass over memory where the caller lends a scratch copy. FP32
 // storage: FP64 steps are bound by the FP64 pipe and 16-bit ones by issue slots as much as by
 // HBM (256^3: 320 against 311 us a step); D3Q19 sets and D2Q9's diagonals across an x wall have
-// no such kernel. In 3D from a million nodes on: below, the state stays in L2 and single steps
-// are as fast (96^3: 18.5 against 21 us; 128^3: 54.6 against 44 us).
+// no such kernel. In 3D from a million nodes on, where the box suits the kernel's tiles: below, the
+// state stays in L2 and single steps are as fast (96^3: 18.5 against 21 us; 128^3: 54.6 against 42).
 bool two_steps_apply(const lbm_params* p) {
     if (p->flow || p->storage != LBM_F32) return false;
-    if (p->lattice == LBM_D3Q7) return (long long)p->nx * p->ny * p->nz >= 1000000;
+    if (p->lattice == LBM_D3Q7)
+        return (long long)p->nx * p->ny * p->nz >= 1000000 && lbm::two_steps_pay_3d(p->nx, p->ny, p->nz);
     return p->lattice == LBM_D2Q5 || (p->lattice == LBM_D2Q9 && !p->wall_x);
 }
 size_t storage_size(int s) { return s == LBM_F64 ? 8 : (s == LBM_F32 ? 4 : 2); }

@@ -18,7 +18,6 @@
 
 namespace lbm {
 
-constexpr int kBlockX = 128;
 
 // Step kernels follow one another in a stream with programmatic dependent launch: the next
 // one's blocks are set up while the last blocks of this one still run (launch_dependents, once
@@ -1670,16 +1669,9 @@ inline dim3 node_grid(const DevParams& P, int& bx) {
     return dim3((P.nx + bx - 1) / bx, P.ny, P.z_hi - P.z_lo);
 }
 
-// Rows of the per-node step and phi kernels: blocks of 128, 96 or 64 nodes of a row, whichever
-// leaves the fewest lanes past its end; single warps in lattices so small that each SM gets at
-// most two (512 x 8 FP64 couple: 5.2 us a step against 8.2). One row per block: with y the same for a whole block the wrap
-// tests of Nbr stay uniform (two-row blocks cost the in-place FP16 step 6 %).
+// Rows of the per-node step and phi kernels.
 inline dim3 step_grid(const DevParams& P, int& bx) {
-    const long long n = (long long)P.nx * P.ny * (P.z_hi - P.z_lo);
-    bx = P.nx >= kBlockX ? kBlockX : (P.nx + 31) / 32 * 32;
-    for (int b : {96, 64})
-        if ((P.nx + b - 1) / b * b < (P.nx + bx - 1) / bx * bx) bx = b;
-    if (n <= 32 * 152 * 2) bx = 32;
+    bx = step_width(P.nx, (long long)P.nx * P.ny * (P.z_hi - P.z_lo));
     return dim3((P.nx + bx - 1) / bx, P.ny, P.z_hi - P.z_lo);
 }
 

@@ -19,6 +19,20 @@ constexpr int kModeAAEven = 0, kModeAAOdd = 1, kModePull = 2;
 // What a kernel whose bounded wait ran out leaves in the context's fault word.
 constexpr unsigned kWaitFault = 0x57414954u;
 
+constexpr int kBlockX = 128;
+
+// Threads of a block of the per-node step and phi kernels, all of one row: 128, 96 or 64, whichever
+// leaves the fewest lanes past the row's end; single warps in lattices so small that each SM gets at
+// most two (512 x 8 FP64 couple: 5.2 us a step against 8.2). One row per block: with y the same for
+// a whole block the wrap tests of Nbr stay uniform (two-row blocks cost the in-place FP16 step 6 %).
+inline int step_width(int nx, long long nodes) {
+    if (nodes <= 32 * 152 * 2) return 32;
+    int bx = nx >= kBlockX ? kBlockX : (nx + 31) / 32 * 32;
+    for (int b : {96, 64})
+        if ((nx + b - 1) / b * b < (nx + bx - 1) / bx * bx) bx = b;
+    return bx;
+}
+
 // Planes (rows, in 2D) a marching block goes through: the count, up to ``most``, for which the
 // waves of blocks over the chip's ``slots`` times the planes each block computes, ``extra`` for
 // the planes around the chunk among them, are fewest.
@@ -31,6 +45,36 @@ inline int march_chunk(long long tiles, int n, long long slots, double extra, in
         if (t <= cost) { cost = t; best = c; }
     }
     return best;
+}
+
+// 3D two-step kernel: a block of 32 x 16 threads, of which the inner 28 x 14 own nodes.
+constexpr int T2X = 32, T2Y = 16, T2IX = T2X - 4, T2IY = T2Y - 2;
+constexpr int kTwoStepsBlocks = 2;                                     // resident on an SM
+
+// Whether two steps a pass take less time than single steps on a D3Q7 lattice without flow. A pass
+// takes the time of the blocks' turns, their threads times the planes they compute, those past the
+// box and around a chunk among them. A single step takes the longest of its memory traffic (less
+// where the L2 holds the state), of its blocks' launches and of its lanes, idle ones among them. Both
+// in ps a node and step, fitted to 130 boxes of 1 to 17 million nodes (two of them come out on the
+// wrong side, by 1.5 %). Single step over
+// two steps a pass, measured: 256^3 1.43, 128^3 1.29, 28x14x4000 2.04, 16x512x128 2.36, 64x64x4096
+// 1.24, 150x84x80 1.01; below one, refused: 57x29x1000 0.85, 64x64x256 0.88, 101^3 0.95, 29x15x2400
+// 0.68, 512x16x128 0.76, 1024x1024x1 0.65, 1024x1x1024 0.15.
+inline bool two_steps_pay_3d(int nx, int ny, int nz) {
+    const double n = double(nx) * ny * nz;
+    const long long tiles = (long long)((nx + T2IX - 1) / T2IX) * ((ny + T2IY - 1) / T2IY), slots = 152 * kTwoStepsBlocks;
+    const int zc = march_chunk(tiles, nz, slots, 2.0);
+    const long long rounds = (tiles * ((nz + zc - 1) / zc) + slots - 1) / slots;
+    const double turns = double(rounds) * slots * T2X * T2Y * (zc + 1.2) / n;
+    const double pass = (n < 1.6e6 ? 5.0 : 3.5) + 8.9 * turns;
+    const int bx = step_width(nx, (long long)n);
+    const double rows = double(ny) * nz * ((nx + bx - 1) / bx) / n;    // blocks a node
+    const double lanes = bx * rows;
+    const double memory = 20.5 + 5.0 * (n < 1.1e6 ? 0.0 : (n < 1.4e6 ? (n - 1.1e6) / 0.3e6 : 1.0));
+    double single = memory * (0.8 + 0.2 * lanes);
+    for (double t : {1015.0 * rows, 17.5 * lanes})
+        if (t > single) single = t;
+    return pass <= single;
 }
 
 // Whether an FP32 two-buffer flow step on D3Q7 sets takes the TMA-staged kernel (given a phi field

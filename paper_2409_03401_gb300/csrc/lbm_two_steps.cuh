@@ -103,10 +103,8 @@ __device__ __forceinline__ bool block_barrier_wait(unsigned b, unsigned parity) 
 }
 
 // 3D: a block of 32 x 16 threads marches along z; its 28 x 14 inner threads own nodes, the
-// outer ring computes the first collision of the tile's neighbours again.
-constexpr int T2X = 32, T2Y = 16, T2IX = T2X - 4, T2IY = T2Y - 2;
-constexpr int kTwoStepsBlocks = 2;
-
+// outer ring computes the first collision of the tile's neighbours again (two_steps_pay_3d: where
+// that is worth it).
 template <class T>
 __global__ void __launch_bounds__(T2X * T2Y, kTwoStepsBlocks)
 two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst, unsigned* fault, int zchunk) {

@@ -1,5 +1,7 @@
-"""The TMA-staged flow step against the fused kernel, bit for bit, in boxes that its rule gives it:
-ragged and whole tiles of 32 x 15 nodes in x and y, many columns of tiles and few, thin boxes."""
+"""Kernels chosen by the shape of a box against the general ones, bit for bit, in boxes that the
+rules give them: for the TMA-staged flow step ragged and whole tiles of 32 x 15 nodes, many columns
+of tiles and few, thin boxes; for two steps a pass in 3D boxes of whole and ragged tiles of 28 x 14
+nodes, narrower than a tile in x, and of few planes."""
 import ctypes
 
 import pytest
@@ -35,3 +37,20 @@ def test_tma_staged_flow_step_matches_the_fused_kernel(shape, collision, wall_z)
     fa, fb = a.fields(), Simulation.attach(p, b.state, 3).fields()
     for k in fa:
         assert torch.equal(fa[k], fb[k]), k
+
+
+@pytest.mark.parametrize("shape", [(28, 14, 2600), (16, 512, 128), (15, 288, 260), (513, 512, 8), (85, 43, 4000)])
+@pytest.mark.parametrize("wall_x,wall_z", [(False, False), (True, True)])
+def test_two_steps_a_pass_match_single_steps(shape, wall_x, wall_z):
+    from paper_2409_03401_gb300 import Simulation, _lib
+    lib = _lib.load()
+    p = LBMParams(*shape, wall_x=wall_x, wall_z=wall_z)
+    f = _inputs(p)
+    a, b = (Simulation(p, *f, device="cuda") for _ in range(2))
+    assert lib.lbm_step_scratch_bytes(ctypes.byref(a._cp)) > 0
+    for n in (4, 1, 7):
+        a.step(n)
+        _lib.check(lib.lbm_step(b._ctx, n), b._ctx)
+        fa, fb = a.fields(), b.fields()
+        for k in fa:
+            assert torch.equal(fa[k], fb[k]), k

@@ -31,3 +31,17 @@ def test_tma_staged_step_where_its_end_tiles_are_few(shape, bgk, mrt):
                                ctypes.byref(ctx)))
         assert lib.lbm_kernels_per_step(ctx) == want, (shape, collision)
         lib.lbm_destroy(ctx)
+
+
+# boxes and the measured time of a single step over that of two steps a pass
+@pytest.mark.parametrize("shape,ratio", [
+    ((256, 256, 256), 1.43), ((128, 128, 128), 1.29), ((128, 96, 96), 1.15), ((150, 84, 80), 1.01), ((28, 14, 4000), 2.04),
+    ((16, 512, 128), 2.36), ((15, 288, 3900), 2.56), ((64, 64, 4096), 1.24), ((512, 512, 8), 1.27), ((85, 43, 4000), 1.16),
+    ((1024, 1024, 1), 0.65), ((1024, 1, 1024), 0.15), ((29, 15, 2400), 0.68), ((29, 15, 38000), 0.85), ((57, 29, 1000), 0.85),
+    ((512, 16, 128), 0.76), ((64, 64, 256), 0.88), ((60, 60, 300), 0.81), ((101, 101, 101), 0.95), ((207, 691, 8), 0.89),
+    ((96, 96, 96), 0.88)])
+def test_two_steps_a_pass_where_the_box_suits_the_tiles(shape, ratio):
+    m, lib = _lib()
+    cp = ctypes.byref(m.make_params(LBMParams(*shape)))
+    want = lib.lbm_copy_bytes(cp) if ratio > 1 else 0
+    assert lib.lbm_step_scratch_bytes(cp) == want, shape
