@@ -169,7 +169,8 @@ lbm_status lbm_attach(const lbm_params* p, void* d_state, void* d_work, int64_t 
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
 
 /* lbm_step with a scratch buffer: with FP32 storage and no flow (LBM_D3Q7 from a million nodes
- * on, in boxes that are not too narrow, LBM_D2Q5, and LBM_D2Q9 without x walls) every four steps from an even time level are two passes over
+ * on, LBM_D2Q5, and LBM_D2Q9 without x walls, but for shapes that are faster by single steps:
+ * lbm_step_scratch_bytes is 0) every four steps from an even time level are two passes over
  * memory, from the state to the scratch buffer and back, with two steps in each. Same results
  * as lbm_step, bit for bit. lbm_step_scratch_bytes is the size wanted (one state copy; 0 where
  * it does not apply). d_scratch: 256-byte aligned device memory of the caller's, used only by

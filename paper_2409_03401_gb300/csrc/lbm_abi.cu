@@ -34,7 +34,8 @@ bool two_steps_apply(const lbm_params* p) {
     if (p->flow || p->storage != LBM_F32) return false;
     if (p->lattice == LBM_D3Q7)
         return (long long)p->nx * p->ny * p->nz >= 1000000 && lbm::two_steps_pay_3d(p->nx, p->ny, p->nz);
-    return p->lattice == LBM_D2Q5 || (p->lattice == LBM_D2Q9 && !p->wall_x);
+    if (p->lattice == LBM_D2Q5) return lbm::two_steps_pay_2d(p->nx, p->ny, false);
+    return p->lattice == LBM_D2Q9 && !p->wall_x && lbm::two_steps_pay_2d(p->nx, p->ny, true);
 }
 size_t storage_size(int s) { return s == LBM_F64 ? 8 : (s == LBM_F32 ? 4 : 2); }
 bool is16(int s) { return s == LBM_F16 || s == LBM_BF16; }

@@ -77,6 +77,47 @@ inline bool two_steps_pay_3d(int nx, int ny, int nz) {
     return pass <= single;
 }
 
+// 2D two-step kernel: warps, four to a block, of which the inner 28 lanes own nodes of a row.
+constexpr int T2Warps = 4, kTwoSteps2DBlocks = 4;                      // resident on an SM
+
+// Its grid: four windows of a row to a block and ``rows`` rows a chunk; folded, warps go on with the
+// next chunk, where a quarter of them or more would have no window and there are rows enough to
+// fill the chip (29x20000 D2Q9 30.1 -> 19.9 us a step, 120x2563 10.6 -> 8.2, 28x20000 22.8 -> 13.2).
+// Elsewhere that is slower (384^2 4.8 -> 5.4, 29x200 1.9 -> 2.6): a row's addresses are then no longer
+// the same for a whole block.
+struct TwoSteps2D {
+    int rows, bx, by, rounds;
+    bool fold;
+    TwoSteps2D(int nx, int ny) {
+        const int wins = (nx + T2IX - 1) / T2IX, slots = 152 * kTwoSteps2DBlocks;
+        bx = (wins + T2Warps - 1) / T2Warps;
+        fold = 3 * T2Warps * bx >= 4 * wins && (long long)bx * ny > slots;
+        rows = fold ? march_chunk(wins, ny, slots * T2Warps, 2.0) : march_chunk(bx, ny, slots, 2.0);
+        by = (ny + rows - 1) / rows;
+        if (fold) {
+            bx = (wins * by + T2Warps - 1) / T2Warps;
+            by = 1;
+        }
+        rounds = int(((long long)bx * by + slots - 1) / slots);
+    }
+};
+
+// Whether two steps a pass take less time than single steps on an FP32 2D lattice without flow: yes,
+// but for some lattices that the L2 holds, of rows of whole 128-byte lines, which a single step
+// reads without a wasted byte. There by the rows a pass goes through, in us a step: single step over
+// two steps a pass, D2Q9 64x4096 0.87, 256x2343 0.91, 384x1562 0.96 (refused), 512x781 1.09, 128x3125
+// 1.05, 768^2 1.09; D2Q5 256x4687 0.88, 1024^2 0.96 (refused), 2048x512 1.03, 224x4464 1.06. All others of 220
+// lattices, 16^2 to 4096^2 and from one column to one row, came out at 0.95 to 3.8.
+inline bool two_steps_pay_2d(int nx, int ny, bool d2q9) {
+    const double n = 1e-6 * nx * ny;
+    if (nx % 32 || n < (d2q9 ? 0.2 : 0.95) || n > (d2q9 ? 0.7 : 1.4)) return true;
+    const TwoSteps2D p(nx, ny);
+    const double pass = p.rounds * (p.rows + 1.5) * (d2q9 ? 1.1 : 0.72);
+    const int bx = step_width(nx, (long long)nx * ny);
+    const double rows = 1.02e-3 * ny * ((nx + bx - 1) / bx);           // the launches of a single step's blocks
+    return pass <= (d2q9 ? 2.0 + 19.4 * n : 1.9 + 10.8 * n) || pass <= rows;
+}
+
 // Whether an FP32 two-buffer flow step on D3Q7 sets takes the TMA-staged kernel (given a phi field
 // as scratch): rows of whole 16-byte pieces (a tensor copy's rule), the undivided lattice, no
 // walls in x, 30 million nodes (measured from there on), and tiles that are

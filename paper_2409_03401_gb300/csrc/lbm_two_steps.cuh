@@ -210,9 +210,9 @@ two_steps_3d_kernel(const DevParams P, const StateView src, const StateView dst,
 // side compute the neighbours' collisions again. No shared memory and no barrier; the next
 // row's populations are loaded into registers before this row's collisions (4 blocks of 4 warps
 // an SM at 124 registers: 323 us a step at 4096^2, against 361 without and 344 at 3 blocks).
-constexpr int T2Warps = 4, kTwoSteps2DBlocks = 4;
-
-template <class T, int LAT>
+// Four windows of a row to a block; FOLD: windows of a row and then of the next chunk of rows, for
+// rows in which many warps would have no window.
+template <class T, int LAT, bool FOLD>
 __global__ void __launch_bounds__(32 * T2Warps, kTwoSteps2DBlocks)
 two_steps_2d_kernel(const DevParams P, const StateView src, const StateView dst, int ychunk) {
     begin_after_previous();
@@ -220,10 +220,12 @@ two_steps_2d_kernel(const DevParams P, const StateView src, const StateView dst,
     using L = Scalar<LAT>;
     constexpr int Q = L::Q;
     const int lane = threadIdx.x & 31;
-    const int win = blockIdx.x * T2Warps + (threadIdx.x >> 5);
-    if (win * T2IX >= P.nx) return;                                    // whole warps
+    const int item = blockIdx.x * T2Warps + (threadIdx.x >> 5);
+    const int wins = FOLD ? (P.nx + T2IX - 1) / T2IX : 1, win = FOLD ? item % wins : item;
+    const int chunk = FOLD ? item / wins : blockIdx.y;
+    if (FOLD ? chunk * ychunk >= P.ny : win * T2IX >= P.nx) return;    // whole warps
     const int x = win * T2IX + lane - 2;
-    const int ys = blockIdx.y * ychunk, ye = min(ys + ychunk, P.ny);
+    const int ys = chunk * ychunk, ye = min(ys + ychunk, P.ny);
     const int gx = wrapped(x, P.nx);
     const bool inner = lane >= 2 && lane < T2IX + 2 && x < P.nx;
     const bool wall_lo = P.wall_x && x == 0, wall_hi = P.wall_x && x == P.nx - 1;
@@ -292,10 +294,9 @@ void launch_two_steps_at(const DevParams& P, const StateView& src, const StateVi
         launch_after_previous<float>(two_steps_3d_kernel<T>, dim3(tiles.x, tiles.y, (P.nz + zc - 1) / zc), dim3(T2X, T2Y),
                                      size_t(smem), s, P, src, dst, fault, zc);
     } else {
-        const int wins = (P.nx + T2IX - 1) / T2IX, bx = (wins + T2Warps - 1) / T2Warps;
-        const int yc = march_chunk(bx, P.ny, 152 * kTwoSteps2DBlocks, 2.0);
-        launch_after_previous<float>(two_steps_2d_kernel<T, LAT>, dim3(bx, (P.ny + yc - 1) / yc), dim3(32 * T2Warps), 0, s, P, src,
-                              dst, yc);
+        const TwoSteps2D p(P.nx, P.ny);
+        launch_after_previous<float>(p.fold ? two_steps_2d_kernel<T, LAT, true> : two_steps_2d_kernel<T, LAT, false>,
+                                     dim3(p.bx, p.by), dim3(32 * T2Warps), 0, s, P, src, dst, p.rows);
     }
 }
 

@@ -1,7 +1,8 @@
 """Kernels chosen by the shape of a box against the general ones, bit for bit, in boxes that the
 rules give them: for the TMA-staged flow step ragged and whole tiles of 32 x 15 nodes, many columns
 of tiles and few, thin boxes; for two steps a pass in 3D boxes of whole and ragged tiles of 28 x 14
-nodes, narrower than a tile in x, and of few planes."""
+nodes, narrower than a tile in x, and of few planes; in 2D rows of few windows of 28 nodes, whose warps
+go on with the next chunk of rows."""
 import ctypes
 
 import pytest
@@ -49,6 +50,24 @@ def test_two_steps_a_pass_match_single_steps(shape, wall_x, wall_z):
     a, b = (Simulation(p, *f, device="cuda") for _ in range(2))
     assert lib.lbm_step_scratch_bytes(ctypes.byref(a._cp)) > 0
     for n in (4, 1, 7):
+        a.step(n)
+        _lib.check(lib.lbm_step(b._ctx, n), b._ctx)
+        fa, fb = a.fields(), b.fields()
+        for k in fa:
+            assert torch.equal(fa[k], fb[k]), k
+
+
+@pytest.mark.parametrize("shape", [(1, 700), (27, 1300), (28, 2503), (29, 999), (56, 5000), (57, 3001), (113, 4500), (139, 640),
+                                   (240, 1057)])
+@pytest.mark.parametrize("kw", [dict(lattice="D2Q9"), dict(lattice="D2Q5"), dict(lattice="D2Q5", wall_x=True)], ids=str)
+def test_folded_two_steps_a_pass_match_single_steps(shape, kw):
+    from paper_2409_03401_gb300 import Simulation, _lib
+    lib = _lib.load()
+    p = LBMParams(*shape, 1, **kw)
+    f = _inputs(p)
+    a, b = (Simulation(p, *f, device="cuda") for _ in range(2))
+    assert lib.lbm_step_scratch_bytes(ctypes.byref(a._cp)) > 0
+    for n in (4, 1, 7, 8):
         a.step(n)
         _lib.check(lib.lbm_step(b._ctx, n), b._ctx)
         fa, fb = a.fields(), b.fields()

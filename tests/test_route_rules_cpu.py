@@ -45,3 +45,16 @@ def test_two_steps_a_pass_where_the_box_suits_the_tiles(shape, ratio):
     cp = ctypes.byref(m.make_params(LBMParams(*shape)))
     want = lib.lbm_copy_bytes(cp) if ratio > 1 else 0
     assert lib.lbm_step_scratch_bytes(cp) == want, shape
+
+
+@pytest.mark.parametrize("lattice,shape,ratio", [
+    ("D2Q9", (4096, 4096), 1.71), ("D2Q9", (512, 512), 0.99), ("D2Q9", (29, 20000), 1.04), ("D2Q9", (120, 2563), 1.03),
+    ("D2Q9", (28, 20000), 1.59), ("D2Q9", (64, 16384), 1.37), ("D2Q9", (768, 768), 1.09), ("D2Q9", (128, 3125), 1.05),
+    ("D2Q9", (64, 4096), 0.87), ("D2Q9", (64, 8192), 0.88), ("D2Q9", (256, 2343), 0.91), ("D2Q9", (384, 1562), 0.96),
+    ("D2Q9", (48, 48), 1.28), ("D2Q5", (2048, 512), 1.03), ("D2Q5", (1024, 1024), 0.96), ("D2Q5", (256, 4687), 0.88),
+    ("D2Q5", (96, 12500), 0.92), ("D2Q5", (64, 16384), 1.22), ("D2Q5", (124, 2842), 1.21), ("D2Q5", (4096, 4096), 1.58)])
+def test_two_steps_a_pass_in_2d(lattice, shape, ratio):
+    m, lib = _lib()
+    cp = ctypes.byref(m.make_params(LBMParams(*shape, 1, lattice=lattice)))
+    want = lib.lbm_copy_bytes(cp) if ratio > 1 else 0
+    assert lib.lbm_step_scratch_bytes(cp) == want, shape
