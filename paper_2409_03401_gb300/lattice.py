@@ -4,6 +4,7 @@
 device, binds them with lbm_init, and forwards lbm_step / lbm_fields / lbm_reduce.
 Every step of the method runs in the sm_103a kernels of liblbm_gb300.so.
 """
+import contextlib
 import ctypes
 
 import torch
@@ -13,6 +14,19 @@ from . import _lib
 
 def _ptr(t):
     return ctypes.c_void_p(t.data_ptr())
+
+
+@contextlib.contextmanager
+def _allocation_beside_captures():
+    """While another stream is captured in the global mode, cudaMalloc fails and ends that capture
+    unless this thread's own mode is relaxed (2); torch relaxes it only for the captured stream."""
+    cuda = ctypes.CDLL("libcuda.so.1")
+    mode = ctypes.c_int(2)
+    cuda.cuThreadExchangeStreamCaptureMode(ctypes.byref(mode))
+    try:
+        yield
+    finally:
+        cuda.cuThreadExchangeStreamCaptureMode(ctypes.byref(mode))
 
 
 def droplet_stats(params, sums):
@@ -151,7 +165,8 @@ class Simulation:
             if torch.cuda.is_current_stream_capturing():
                 return None
             try:
-                return torch.empty(self._scratch_bytes, dtype=torch.uint8, device=self.device)
+                with _allocation_beside_captures():
+                    return torch.empty(self._scratch_bytes, dtype=torch.uint8, device=self.device)
             except torch.cuda.OutOfMemoryError:
                 return None
 
