@@ -138,10 +138,16 @@ class Simulation:
     def real_dtype(self):
         return torch.float64 if self.params.storage == "f64" else torch.float32
 
-    def step(self, n=1, graph=False):
+    def step(self, n=1, graph=False, scratch=True):
         """Advance n steps; ``graph=True`` replays a captured CUDA graph of two steps (needs a
-        created stream, e.g. Simulation(..., stream=torch.cuda.Stream()))."""
-        scratch = None if graph or n < 4 else self._scratch()
+        created stream, e.g. Simulation(..., stream=torch.cuda.Stream())).
+
+        FP32 lattices without flow that lbm_step_scratch advances two steps a pass borrow memory for
+        it, for each call of four steps or more: one more state copy at the peak, at most an eighth
+        of the device, which stays in torch's pool afterwards. ``scratch=False`` borrows none and
+        takes single steps; so does ``graph=True``, and every later call once torch had no memory
+        for it. The results are the same."""
+        scratch = self._scratch() if scratch and not graph and n >= 4 else None
         if scratch is not None:
             _lib.check(self.lib.lbm_step_scratch(self._ctx, int(n), _ptr(scratch), scratch.numel()), self._ctx)
             return self
@@ -153,10 +159,12 @@ class Simulation:
         """One state copy from torch's allocator for lbm_step_scratch, on the simulation's stream
         (returned to the allocator after the call, which reuses it in stream order), or None
         where the library takes no scratch, while the stream is being captured, for a copy above
-        an eighth of the device's memory, or when the memory is not there."""
+        an eighth of the device's memory, or once the memory was not there: torch frees its cached
+        blocks and synchronises before it says so, which no call should repeat."""
         if not hasattr(self, "_scratch_bytes"):
             b = self.lib.lbm_step_scratch_bytes(ctypes.byref(self._cp))
-            if b and b > torch.cuda.get_device_properties(self.device).total_memory // 8:
+            if b and (b > torch.cuda.get_device_properties(self.device).total_memory // 8
+                      or not isinstance(self.stream, torch.cuda.Stream)):
                 b = 0
             self._scratch_bytes = b
         if not self._scratch_bytes:
@@ -168,6 +176,7 @@ class Simulation:
                 with _allocation_beside_captures():
                     return torch.empty(self._scratch_bytes, dtype=torch.uint8, device=self.device)
             except torch.cuda.OutOfMemoryError:
+                self._scratch_bytes = 0
                 return None
 
     def fields(self, names=_lib.FIELDS):

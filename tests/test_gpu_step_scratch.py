@@ -42,3 +42,32 @@ def test_step_while_another_stream_is_captured():
     assert a.t == b.t == 9
     _same(a, b)
 
+
+def test_no_memory_is_asked_for_once(monkeypatch):
+    a, b = _sim(), _sim()
+    empty, asked = torch.empty, []
+
+    def refuse(*size, **kw):
+        if kw.get("dtype") == torch.uint8:
+            asked.append(size)
+            raise torch.cuda.OutOfMemoryError("none left")
+        return empty(*size, **kw)
+
+    monkeypatch.setattr(torch, "empty", refuse)
+    a.step(8).step(5).step(4)
+    monkeypatch.undo()
+    assert len(asked) == 1
+    b.step(17)
+    _same(a, b)
+
+
+def test_scratch_can_be_declined():
+    a, b = _sim(), _sim()
+    torch.cuda.synchronize()
+    torch.cuda.reset_peak_memory_stats()
+    before = torch.cuda.memory_allocated()
+    a.step(8, scratch=False)
+    assert torch.cuda.max_memory_allocated() == before
+    b.step(8)
+    assert torch.cuda.max_memory_allocated() > before
+    _same(a, b)
