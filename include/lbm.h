@@ -149,7 +149,9 @@ size_t lbm_work_bytes(const lbm_params* p);
  * p_h = 0, u = 0 shifted by the initial forcing. d_phi0, d_cA0, d_cB0 are FP64 device
  * arrays of nx*ny*nz values, x fastest; they are read during the call's kernel and may
  * be freed once the stream has passed it. d_state (lbm_state_bytes) and d_work
- * (lbm_work_bytes) must be 256-byte aligned and stay valid until lbm_destroy.
+ * (lbm_work_bytes) must be 256-byte aligned and stay valid until lbm_destroy. A work buffer
+ * belongs to one context: steps, fields and sums all write it, so two contexts may share one
+ * only if their work never overlaps in time, on whatever streams.
  * On success *out receives a new context (time 0). */
 lbm_status lbm_init(const lbm_params* p, void* d_state, void* d_work,
                     const double* d_phi0, const double* d_cA0, const double* d_cB0,
@@ -163,9 +165,9 @@ lbm_status lbm_attach(const lbm_params* p, void* d_state, void* d_work, int64_t 
 
 /* Advance nsteps >= 0 coupled time steps (§3): one fused collide-and-stream kernel per
  * step; with flow, all but LBM_BF16 and FP32 lattices of 600,000 nodes and more with two copies
- * and LBM_D3Q7 scalars add a phi pass for the capillary stencil, and FP32 lattices of 30
- * million nodes and more a pass for phi of their x and y ends (lbm_kernels_per_step). The
- * passes use the phi field of the work buffer. Asynchronous. */
+ * and LBM_D3Q7 scalars add a phi pass for the capillary stencil, and FP32 boxes of 30 million
+ * nodes and more with few nodes at their ends a pass for phi of those (lbm_kernels_per_step).
+ * The passes write the phi field of the work buffer. Asynchronous. */
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
 
 /* lbm_step with a scratch buffer: with FP32 storage and no flow (LBM_D3Q7 from a million nodes
@@ -174,7 +176,8 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
  * memory, from the state to the scratch buffer and back, with two steps in each. Same results
  * as lbm_step, bit for bit. lbm_step_scratch_bytes is the size wanted (one state copy; 0 where
  * it does not apply). d_scratch: 256-byte aligned device memory of the caller's, used only by
- * the work this call queues; NULL or fewer bytes take lbm_step's path, as do steps recorded by
+ * the work this call queues (where the call is captured, by every replay: it must outlive the
+ * graph); NULL or fewer bytes take lbm_step's path, as do steps recorded by
  * lbm_profile_begin and slabs. Asynchronous. No counterpart in the paper. */
 size_t lbm_step_scratch_bytes(const lbm_params* p);
 lbm_status lbm_step_scratch(lbm_ctx* ctx, int nsteps, void* d_scratch, size_t scratch_bytes);
@@ -182,7 +185,9 @@ lbm_status lbm_step_scratch(lbm_ctx* ctx, int nsteps, void* d_scratch, size_t sc
 /* Advance nsteps coupled time steps by replaying a CUDA graph of two steps (captured on the
  * first call from an even time level, after one plain pair of steps; kept until
  * lbm_destroy): the same kernels and results as lbm_step, bit for bit, with one launch per
- * two steps, for lattices small enough that launch overhead shows. The context's stream must
+ * two steps, for lattices small enough that launch overhead shows. It takes no scratch buffer:
+ * where lbm_step_scratch_bytes is not 0, lbm_step_scratch is faster (256^3 297 against 423 us a
+ * step). The context's stream must
  * be one the caller created (the legacy and per-thread default streams cannot be captured:
  * LBM_ERR_ARG). The replayed graph holds the buffers bound at lbm_init/lbm_attach; steps run
  * this way are not recorded by lbm_profile_begin. No counterpart in the paper. */

@@ -145,8 +145,8 @@ class Simulation:
         FP32 lattices without flow that lbm_step_scratch advances two steps a pass borrow memory for
         it, for each call of four steps or more: one more state copy at the peak, at most an eighth
         of the device, which stays in torch's pool afterwards. ``scratch=False`` borrows none and
-        takes single steps; so does ``graph=True``, and every later call once torch had no memory
-        for it. The results are the same."""
+        takes single steps (256^3: 423 us a step against 297); so do ``graph=True`` and every later
+        call once torch had no memory for it. The results are the same."""
         scratch = self._scratch() if scratch and not graph and n >= 4 else None
         if scratch is not None:
             _lib.check(self.lib.lbm_step_scratch(self._ctx, int(n), _ptr(scratch), scratch.numel()), self._ctx)
