@@ -288,7 +288,8 @@ int read_mode(const lbm_ctx* c) {
 }
 // Whether a flow step of the two-buffer layout runs as the fused kernel: FP32 storage from
 // 600,000 nodes on, BF16 storage, and slabs (whose ghost phi it reads in place). The others take
-// a phi pass and the per-node pull step, the same fields bit for bit. The fused kernel computes
+// a phi pass and the per-node pull step, the same fields bit for bit (but for the last place of phi
+// below 1e-27, far from any droplet, where products underflow on the way). The fused kernel computes
 // phi of its halo again (a third more): that saves HBM traffic, but FP16 and FP64 storage pay
 // for it in issue slots and on the FP64 pipe (512^3 FP16 8.01 ms against 7.29 for the two
 // passes, 64^3 27 against 21 us; FP64 128^3 2.45 against 2.16 ms), and in lattices that stay in

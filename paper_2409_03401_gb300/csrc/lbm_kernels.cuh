@@ -783,8 +783,14 @@ __device__ __forceinline__ void step_node(const A& ad, const DevParams& P, const
 // ------------------------------------------------------------------------------------
 // One coupled step per node. With flow the phi field of this step must already be in
 // phi_field (phi pass); MODE AA_* works in place on ``st``, PULL reads ``st`` and writes ``out``.
+// Blocks an SM that an instance is held to (0: the compiler's own choice): the odd FP32 MRT step in
+// place takes 101 registers, four blocks, by itself (256^3 in place 1294 us a step, with five 1222).
+template <class T, int LAT, int MODE, int COLL>
+constexpr int step_min_blocks() {
+    return std::is_same<T, float>::value && LAT == LAT_D3Q7 && MODE == AA_ODD && COLL == 2 ? 5 : 0;
+}
 template <class T, int LAT, bool FLOW, int MODE, int COLL>
-__global__ void __launch_bounds__(kBlockX)
+__global__ void __launch_bounds__(kBlockX, (step_min_blocks<T, LAT, MODE, COLL>()))
 step_kernel(const DevParams P, const StateView st, const StateView out, const typename RealOf<T>::type* phi_field) {
     using R = typename RealOf<T>::type;
     begin_after_previous();
