@@ -31,9 +31,9 @@ N = 512
 # four rest populations g_0, h^A_0, h^B_0, f_0 in FP32 (36 x 2 B + 4 x 4 B = 88 B each way)
 ALG_BYTES_PER_NODE = {"f32": 320.0, "f16": 176.0, "bf16": 176.0, "f64": 640.0}
 # DRAM bytes (read + write) per node of one FP32 step, from an ncu capture at 320^3:
-# flow_tma_kernel 189.6 + 158.7, rim_phi_kernel 15.3 + 0.15 (of the x and y ends: 320/512 of
+# flow_tma_kernel 188.5 + 158.6, rim_phi_kernel 15.3 + 0.2 (of the x and y ends: 320/512 of
 # it at 512^3). Set to None whenever the kernels change until they are captured again.
-NCU_DRAM_BYTES_PER_NODE_F32 = 189.6 + 158.7 + 15.4 * 320 / 512
+NCU_DRAM_BYTES_PER_NODE_F32 = 188.5 + 158.6 + 15.5 * 320 / 512
 
 
 def parse():
